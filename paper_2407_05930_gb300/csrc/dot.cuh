@@ -82,92 +82,121 @@ __device__ __forceinline__ void dot_finalize_rhs(const DotArgs& d, const double*
 }
 
 // Block + grid reduction.  part[q] is this thread's partial for column
-// c0 + q (zero when !has_cols).  Threads of one row slot are S consecutive
-// lanes; when S is a power of two <= 32 the row slots of a warp are first
-// combined with xor shuffles (lanes l, l^S, l^2S, ... share their columns),
-// so shared memory holds one partial per warp and column; otherwise every
-// slot gets its own line.  Shared scratch (dynamic): dot_smem_doubles(...).
-// Every sum runs in a fixed assignment of threads to terms, so the order of
-// additions, and the result, never varies from run to run.
+// c0 + q (zero when !has_cols).  Every sum runs in a fixed assignment of
+// threads to terms, so the order of additions, and the result, never varies
+// from run to run.  Shared scratch (dynamic): dot_smem_doubles(...).
+//
+// What bounds it: FP64 adds issue at 2 lanes per clock per SM here (16 cycles
+// a warp instruction) and one dependent add takes longer than a shared load,
+// so the tail of a fused dot is the number of FP64 add instructions per warp
+// plus the chains of dependent adds, not the bytes.  Hence: a warp combines
+// its row slots by halving exchanges (lane pairs swap half of their columns,
+// so 8 columns over 32 lanes take 4 + 2 + 1 + 1 + 1 = 9 adds a lane, not
+// 8 x 5 = 40), and every later stage sums a few interleaved chains.
+// Measured on whole solves to 1e-12: FP64 2D 64x64 (C = 2, three dots an
+// iteration) 4.05 -> 2.96 ms, mixed 256^3 (C = 8) 107.1 -> 103.9 ms, against
+// full butterflies of every column and one thread per column summing up to 128
+// slices.
+__host__ __device__ inline bool dot_shuffles(int S) { return S > 0 && (S & (S - 1)) == 0 && S <= 32; }
+
+// Lines of per-column partials a block leaves in shared memory: one per warp
+// when the S lanes of a row slot divide a warp, else one per row slot.
+__host__ __device__ inline int dot_lines(int S, int rows_pb) { return dot_shuffles(S) ? kBlock / 32 : rows_pb; }
+
 __host__ __device__ inline int dot_smem_doubles(int S, int rows_pb, int C) {
-  const bool pow2 = S > 0 && (S & (S - 1)) == 0 && S <= 32;
-  const int lines = pow2 ? kBlock / 32 : rows_pb;
-  return lines * C + kBlock + C;
+  return dot_lines(S, rows_pb) * C + kBlock + C;
 }
 
-template <int CPT>
-__device__ __forceinline__ void block_dot(const DotArgs& d, double (&part)[CPT], int c0, bool has_cols,
-                                          int rloc, int rows_pb, int S, int C, double* sm, int slot, int nslots,
-                                          double* partials, unsigned* ticket) {
-  const bool pow2 = (S & (S - 1)) == 0 && S <= 32;
-  int lines;
-  if (pow2) {
-    for (int off = S; off < 32; off <<= 1) {
+// Steps K.. of the halving exchange over the lanes lane ^ (S << K): v[0 .. NV)
+// holds columns sub .. sub + NV - 1 of the thread's CPT.  `dup`: this lane's
+// last value is also held by a lower lane.
+template <int NV, int CPT>
+__device__ __forceinline__ void dot_exchange(double (&v)[CPT], int off, int lane, int& sub, bool& dup) {
+  if constexpr (NV > 1) {
+    if (off >= 32) return;
+    constexpr int H = NV / 2;
+    const bool up = (lane & off) != 0;
 #pragma unroll
-      for (int q = 0; q < CPT; ++q) part[q] += __shfl_xor_sync(0xffffffffu, part[q], off);
+    for (int q = 0; q < H; ++q) {
+      const double send = up ? v[q] : v[q + H];
+      const double keep = up ? v[q + H] : v[q];
+      v[q] = keep + __shfl_xor_sync(0xffffffffu, send, off);
     }
-    lines = kBlock / 32;
-    const int lane = threadIdx.x & 31;
-    if (has_cols && lane < S) {
-#pragma unroll
-      for (int q = 0; q < CPT; ++q) sm[(threadIdx.x >> 5) * C + c0 + q] = part[q];
-    }
+    if (up) sub += H;
+    dot_exchange<H, CPT>(v, off << 1, lane, sub, dup);
   } else {
-    lines = rows_pb;
-    if (has_cols) {
+    for (; off < 32; off <<= 1) {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], off);
+      if (lane & off) dup = true;
+    }
+  }
+}
+
+// The block's threads' partials as lines of C columns in sm (unsynchronised).
+template <int CPT>
+__device__ __forceinline__ void dot_block_lines(double (&part)[CPT], int c0, bool has_cols, int rloc, int S, int C,
+                                                double* sm) {
+  if (dot_shuffles(S)) {
+    const int lane = threadIdx.x & 31;
+    int sub = 0;
+    bool dup = false;
+    dot_exchange<CPT, CPT>(part, S, lane, sub, dup);
+    // log2(32 / S) halvings leave max(1, CPT S / 32) columns per lane
+    const int left = CPT * S > 32 ? CPT * S / 32 : 1;
+    if (has_cols && !dup) {
+      double* line = sm + (threadIdx.x >> 5) * C + c0 + sub;
 #pragma unroll
-      for (int q = 0; q < CPT; ++q) sm[rloc * C + c0 + q] = part[q];
+      for (int q = 0; q < CPT; ++q)
+        if (q < left) line[q] = part[q];
     }
+  } else if (has_cols) {
+#pragma unroll
+    for (int q = 0; q < CPT; ++q) sm[rloc * C + c0 + q] = part[q];
   }
-  __syncthreads();
-  const int slices = blockDim.x / C;  // C <= 256 = blockDim
-  double* red = sm + lines * C;       // [slices][C], <= 256 doubles
-  if ((int)threadIdx.x < slices * C) {
-    const int c = threadIdx.x % C, sl = threadIdx.x / C;
-    double t0 = 0.0, t1 = 0.0;
+}
+
+// out[c] = sum of `count` lines of src (stride C; GLOBAL: written by other
+// blocks, read through L2), for the whole block: thread t sums the lines
+// t / C, t / C + slices, ... of column t % C in four chains, then the slices
+// are added in shared memory (red: kBlock doubles) by four chains again.
+// Synchronises before out may be read.
+template <bool GLOBAL>
+__device__ __forceinline__ void dot_sum_lines(const double* src, int count, int C, double* red, double* out) {
+  const int c = threadIdx.x % C, sl = threadIdx.x / C;
+  auto ld = [&](int r) { return GLOBAL ? __ldcg(src + (int64_t)r * C + c) : src[r * C + c]; };
+  // few lines: one thread per column, no second stage
+  const int slices = count <= 8 ? 1 : min((int)blockDim.x / C, count);
+  if (sl < slices) {
+    double t[4] = {0.0, 0.0, 0.0, 0.0};
     int r = sl;
-    for (; r + slices < lines; r += 2 * slices) {
-      t0 += sm[r * C + c];
-      t1 += sm[(r + slices) * C + c];
+    for (; r + 3 * slices < count; r += 4 * slices) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) t[u] += ld(r + u * slices);
     }
-    if (r < lines) t0 += sm[r * C + c];
-    red[sl * C + c] = t0 + t1;
+#pragma unroll
+    for (int u = 0; u < 3; ++u)
+      if (r + u * slices < count) t[u] += ld(r + u * slices);
+    const double v = (t[0] + t[1]) + (t[2] + t[3]);
+    if (slices == 1)
+      out[c] = v;
+    else
+      red[sl * C + c] = v;
+  }
+  // halve the slices until one is left: log2(slices) dependent adds
+  for (int n = slices; n > 1;) {
+    const int h = (n + 1) >> 1;
+    __syncthreads();
+    if (sl < n - h) red[sl * C + c] += red[(sl + h) * C + c];
+    n = h;
+  }
+  if (slices > 1) {
+    if (sl == 0) out[c] = red[c];
   }
   __syncthreads();
-  for (int c = threadIdx.x; c < C; c += blockDim.x) {
-    double t = 0.0;
-    for (int sl = 0; sl < slices; ++sl) t += red[sl * C + c];
-    partials[(int64_t)slot * C + c] = t;
-  }
-  __threadfence();
-  __syncthreads();
-  __shared__ unsigned is_last;
-  if (threadIdx.x == 0) is_last = (atomicAdd(ticket, 1u) == (unsigned)nslots - 1u) ? 1u : 0u;
-  __syncthreads();
-  if (!is_last) return;
-  __threadfence();
-  if ((int)threadIdx.x < slices * C) {
-    const int c = threadIdx.x % C, sl = threadIdx.x / C;
-    const int nblk = nslots;
-    double t0 = 0.0, t1 = 0.0, t2 = 0.0, t3 = 0.0;
-    int b = sl;
-    for (; b + 3 * slices < nblk; b += 4 * slices) {
-      t0 += __ldcg(partials + (int64_t)b * C + c);
-      t1 += __ldcg(partials + (int64_t)(b + slices) * C + c);
-      t2 += __ldcg(partials + (int64_t)(b + 2 * slices) * C + c);
-      t3 += __ldcg(partials + (int64_t)(b + 3 * slices) * C + c);
-    }
-    for (; b < nblk; b += slices) t0 += __ldcg(partials + (int64_t)b * C + c);
-    red[sl * C + c] = (t0 + t1) + (t2 + t3);
-  }
-  __syncthreads();
-  double* colsum = sm;  // [C]
-  for (int c = threadIdx.x; c < C; c += blockDim.x) {
-    double t = 0.0;
-    for (int sl = 0; sl < slices; ++sl) t += red[sl * C + c];
-    colsum[c] = t;
-  }
-  __syncthreads();
+}
+
+// The CG scalars of every column, then of every right-hand side.
+__device__ __forceinline__ void dot_finalize(const DotArgs& d, const double* colsum, int C) {
   for (int c = threadIdx.x; c < C; c += blockDim.x) {
     double t = colsum[c];
     if (d.coupled) {  // one CG per RHS: the sum over its blocks, in block order
@@ -177,8 +206,34 @@ __device__ __forceinline__ void block_dot(const DotArgs& d, double (&part)[CPT],
     }
     dot_finalize_column(d, c, t);
   }
+  if (d.final == FIN_CONV || d.final == FIN_STORE_BN) {
+    __syncthreads();
+    dot_finalize_rhs(d, colsum);
+  }
+}
+
+template <int CPT>
+__device__ __forceinline__ void block_dot(const DotArgs& d, double (&part)[CPT], int c0, bool has_cols,
+                                          int rloc, int rows_pb, int S, int C, double* sm, int slot, int nslots,
+                                          double* partials, unsigned* ticket) {
+  const int lines = dot_lines(S, rows_pb);
+  double* red = sm + lines * C;
+  dot_block_lines<CPT>(part, c0, has_cols, rloc, S, C, sm);
   __syncthreads();
-  dot_finalize_rhs(d, colsum);
+  dot_sum_lines<false>(sm, lines, C, red, partials + (int64_t)slot * C);
+  __shared__ unsigned is_last;
+  if (threadIdx.x == 0) {
+    // the block's stores, made visible to this thread by the barrier, are
+    // released with its arrival (cumulativity), and acquired by the last block
+    __threadfence();
+    is_last = (atomicAdd(ticket, 1u) == (unsigned)nslots - 1u) ? 1u : 0u;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!is_last) return;
+  double* colsum = sm;  // [C] (the line area is free now)
+  dot_sum_lines<true>(partials, nslots, C, red, colsum);
+  dot_finalize(d, colsum, C);
   if (threadIdx.x == 0) *ticket = 0u;
   __syncthreads();  // the block may go on to reuse the shared scratch
 }
@@ -188,74 +243,34 @@ __device__ __forceinline__ void block_dot(const DotArgs& d, double (&part)[CPT],
 template <int CPT>
 __device__ __forceinline__ void block_dot2(const DotArgs& d, double (&part)[CPT], int c0, bool has_cols, int rloc,
                                            int rows_pb, int S, int C, double* sm, int slot, const BDot& bd) {
-  const bool pow2 = (S & (S - 1)) == 0 && S <= 32;
-  int lines;
-  if (pow2) {
-    for (int off = S; off < 32; off <<= 1) {
-#pragma unroll
-      for (int q = 0; q < CPT; ++q) part[q] += __shfl_xor_sync(0xffffffffu, part[q], off);
-    }
-    lines = kBlock / 32;
-    const int lane = threadIdx.x & 31;
-    if (has_cols && lane < S) {
-#pragma unroll
-      for (int q = 0; q < CPT; ++q) sm[(threadIdx.x >> 5) * C + c0 + q] = part[q];
-    }
-  } else {
-    lines = rows_pb;
-    if (has_cols) {
-#pragma unroll
-      for (int q = 0; q < CPT; ++q) sm[rloc * C + c0 + q] = part[q];
-    }
-  }
+  const int lines = dot_lines(S, rows_pb);
+  double* red = sm + lines * C;
+  dot_block_lines<CPT>(part, c0, has_cols, rloc, S, C, sm);
   __syncthreads();
-  const int slices = blockDim.x / C;
-  double* red = sm + lines * C;  // [slices][C]
-  // sum `count` lines of `src` (stride C) into red, then red over slices -> out
-  auto reduce_lines = [&](const double* src, int count, bool global_src, double* out) {
-    if ((int)threadIdx.x < slices * C) {
-      const int c = threadIdx.x % C, sl = threadIdx.x / C;
-      double t0 = 0.0, t1 = 0.0;
-      int r = sl;
-      for (; r + slices < count; r += 2 * slices) {
-        t0 += global_src ? __ldcg(src + (int64_t)r * C + c) : src[r * C + c];
-        t1 += global_src ? __ldcg(src + (int64_t)(r + slices) * C + c) : src[(r + slices) * C + c];
-      }
-      if (r < count) t0 += global_src ? __ldcg(src + (int64_t)r * C + c) : src[r * C + c];
-      red[sl * C + c] = t0 + t1;
-    }
-    __syncthreads();
-    for (int c = threadIdx.x; c < C; c += blockDim.x) {
-      double t = 0.0;
-      for (int sl = 0; sl < slices; ++sl) t += red[sl * C + c];
-      out[c] = t;
-    }
-  };
-  reduce_lines(sm, lines, false, bd.partials + (int64_t)slot * C);
-  __threadfence();
-  __syncthreads();
+  dot_sum_lines<false>(sm, lines, C, red, bd.partials + (int64_t)slot * C);
   __shared__ unsigned last_chunk, last_all;
   const int chunk = slot >> 5;
   const int nch = (bd.nslots + 31) >> 5;
   const int in_chunk = min(32, bd.nslots - chunk * 32);
-  if (threadIdx.x == 0) last_chunk = (atomicAdd(bd.chunk_tickets + chunk, 1u) == (unsigned)in_chunk - 1u) ? 1u : 0u;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last_chunk = (atomicAdd(bd.chunk_tickets + chunk, 1u) == (unsigned)in_chunk - 1u) ? 1u : 0u;
+    __threadfence();
+  }
   __syncthreads();
   if (!last_chunk) return;
-  __threadfence();
-  reduce_lines(bd.partials + (int64_t)chunk * 32 * C, in_chunk, true, bd.chunk_partials + (int64_t)chunk * C);
-  if (threadIdx.x == 0) bd.chunk_tickets[chunk] = 0u;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) last_all = (atomicAdd(bd.ticket, 1u) == (unsigned)nch - 1u) ? 1u : 0u;
+  dot_sum_lines<true>(bd.partials + (int64_t)chunk * 32 * C, in_chunk, C, red, bd.chunk_partials + (int64_t)chunk * C);
+  if (threadIdx.x == 0) {
+    bd.chunk_tickets[chunk] = 0u;
+    __threadfence();
+    last_all = (atomicAdd(bd.ticket, 1u) == (unsigned)nch - 1u) ? 1u : 0u;
+    __threadfence();
+  }
   __syncthreads();
   if (!last_all) return;
-  __threadfence();
-  double* colsum = sm;  // [C] (the line area is free now)
-  reduce_lines(bd.chunk_partials, nch, true, colsum);
-  __syncthreads();
-  for (int c = threadIdx.x; c < C; c += blockDim.x) dot_finalize_column(d, c, colsum[c]);
-  __syncthreads();
-  dot_finalize_rhs(d, colsum);
+  double* colsum = sm;
+  dot_sum_lines<true>(bd.chunk_partials, nch, C, red, colsum);
+  dot_finalize(d, colsum, C);
   if (threadIdx.x == 0) *bd.ticket = 0u;
   __syncthreads();
 }
