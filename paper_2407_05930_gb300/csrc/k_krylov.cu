@@ -21,14 +21,20 @@ namespace {
 constexpr int kJChunk = 8;  // vectors of a set per pass over W
 
 // part[(blk * J + j) * C + c] = sum over this block's rows of V_j[row][c % Cv] * W[row][c].
+// A thread keeps kJChunk sums of one column.  With C dividing a warp the lanes
+// of a column combine by the halving exchange of dot.cuh (they swap half of
+// their kJChunk sums), and one barrier per chunk hands the warps' lines to
+// the threads that add them; otherwise every row slot leaves its line.
 __global__ void __launch_bounds__(kBlock) mdot_partial_kernel(const double* __restrict__ V, int64_t vstride,
                                                               int32_t Cv, int32_t J, const double* __restrict__ W,
                                                               int64_t rows, int32_t C, double* __restrict__ part) {
-  __shared__ double sm[kBlock];
+  __shared__ double sm[kJChunk * kBlock];  // [line][u][column]
   const int rpb = kBlock / C;  // rows per block step
   const int col = threadIdx.x % C, rl = threadIdx.x / C;
   const bool act = rl < rpb;
   const int vc = col % Cv;
+  const bool shuffles = dot_shuffles(C);
+  const int lines = dot_lines(C, rpb);
   for (int j0 = 0; j0 < J; j0 += kJChunk) {
     double acc[kJChunk];
 #pragma unroll
@@ -41,27 +47,64 @@ __global__ void __launch_bounds__(kBlock) mdot_partial_kernel(const double* __re
           if (j0 + u < J) acc[u] = fma(V[(int64_t)(j0 + u) * vstride + row * Cv + vc], w, acc[u]);
       }
     }
-    for (int u = 0; u < kJChunk && j0 + u < J; ++u) {
-      sm[threadIdx.x] = acc[u];
-      __syncthreads();
-      if (threadIdx.x < C) {
-        double s = 0.0;
-        for (int r = 0; r < rpb; ++r) s += sm[r * C + threadIdx.x];
-        part[((int64_t)blockIdx.x * J + j0 + u) * C + threadIdx.x] = s;
+    __syncthreads();  // the previous chunk's lines have been read
+    if (shuffles) {
+      int sub = 0;
+      bool dup = false;
+      dot_exchange<kJChunk, kJChunk>(acc, C, threadIdx.x & 31, sub, dup);
+      const int left = kJChunk * C > 32 ? kJChunk * C / 32 : 1;
+      double* line = sm + (threadIdx.x >> 5) * kJChunk * C + sub * C + col;
+#pragma unroll
+      for (int u = 0; u < kJChunk; ++u)
+        if (!dup && u < left) line[u * C] = acc[u];
+    } else if (act) {
+#pragma unroll
+      for (int u = 0; u < kJChunk; ++u) sm[rl * kJChunk * C + u * C + col] = acc[u];
+    }
+    __syncthreads();
+    const int nu = min(kJChunk, J - j0) * C;
+    for (int t = threadIdx.x; t < nu; t += kBlock) {
+      double s[4] = {0.0, 0.0, 0.0, 0.0};
+      int r = 0;
+      for (; r + 4 <= lines; r += 4) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s[q] += sm[(r + q) * kJChunk * C + t];
       }
-      __syncthreads();
+      for (; r < lines; ++r) s[0] += sm[r * kJChunk * C + t];
+      part[((int64_t)blockIdx.x * J + j0) * C + t] = (s[0] + s[1]) + (s[2] + s[3]);
     }
   }
 }
 
-// H[j * C + c] = sum over blocks (in block order) of the partials.
-__global__ void mdot_final_kernel(const double* __restrict__ part, int32_t nblk, int32_t J, int32_t C,
-                                  double* __restrict__ H) {
-  for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < J * C; t += gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int b = 0; b < nblk; ++b) s += part[(int64_t)b * J * C + t];
-    H[t] = s;
+// H[t] = sum over blocks of part[b * n + t], n = J * C.  A block serves
+// kFinalCols consecutive sums with kBlock / kFinalCols threads each (their
+// terms strided, then halved in shared memory).  One thread per sum walked up
+// to 608 dependent adds, 110 us a call and two thirds of a GMRES step at 64^3,
+// s = 3; with the exchanges above the solve to 1e-12 went from 22.0 to 12.8 ms.
+constexpr int kFinalCols = 8;
+__global__ void __launch_bounds__(kBlock) mdot_final_kernel(const double* __restrict__ part, int32_t nblk, int32_t n,
+                                                            double* __restrict__ H) {
+  __shared__ double sm[kBlock];
+  constexpr int kSlices = kBlock / kFinalCols;
+  const int t = blockIdx.x * kFinalCols + threadIdx.x % kFinalCols;
+  const int sl = threadIdx.x / kFinalCols;
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+  if (t < n) {
+    int b = sl;
+    for (; b + 3 * kSlices < nblk; b += 4 * kSlices) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) s[q] += part[(int64_t)(b + q * kSlices) * n + t];
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+      if (b + q * kSlices < nblk) s[q] += part[(int64_t)(b + q * kSlices) * n + t];
   }
+  sm[threadIdx.x] = (s[0] + s[1]) + (s[2] + s[3]);
+  for (int h = kSlices / 2; h >= 1; h >>= 1) {
+    __syncthreads();
+    if (sl < h) sm[threadIdx.x] += sm[threadIdx.x + h * kFinalCols];
+  }
+  if (sl == 0 && t < n) H[t] = sm[threadIdx.x];
 }
 
 // W[row][c] += sign * sum_j V_j[row][c % Cv] * H[j * C + c]  (j in order).
@@ -104,7 +147,7 @@ void launch_mdot(const double* V, int64_t vstride, int32_t Cv, int32_t J, const 
   const int g = mdot_blocks(rows, C);
   count_launch(2);
   mdot_partial_kernel<<<g, kBlock, 0, st>>>(V, vstride, Cv, J, W, rows, C, part);
-  mdot_final_kernel<<<std::max(1, (J * C + 255) / 256), 256, 0, st>>>(part, g, J, C, H);
+  mdot_final_kernel<<<(J * C + kFinalCols - 1) / kFinalCols, kBlock, 0, st>>>(part, g, J * C, H);
 }
 
 void launch_maxpy(const double* V, int64_t vstride, int32_t Cv, int32_t J, const double* H, double sign, double* W,
