@@ -324,11 +324,11 @@ static void add_coarse(Batch* B, std::vector<BLaunch>& plan, VecType vt, const s
   L.xt = vt;
   std::vector<BItem> items;
   for (size_t i = 0; i < args.size(); ++i)
-    for (int r = 0; r < args[i].n; r += 32) {
+    for (int r = 0; r < args[i].n; r += kCoarseItemRows) {
       BItem it;
       it.arg = (int32_t)i;
       it.first_slot = r;
-      it.row_end = std::min(args[i].n, r + 32);
+      it.row_end = std::min(args[i].n, r + kCoarseItemRows);
       it.slot = 0;
       items.push_back(it);
     }

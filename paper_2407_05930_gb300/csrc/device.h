@@ -389,6 +389,7 @@ void launch_spmm_batch(ValType mt, VecType xt, VecType ot, int cpt, int kl, bool
                        size_t smem, cudaStream_t st);
 void launch_vec_batch(int op, VecType vt, int cpt, const UpdArgs* args, const BItem* items, int32_t n_items,
                       const BDot* dots, size_t smem, cudaStream_t st);
+constexpr int kCoarseItemRows = 4;  // rows of one item of the batched coarsest solve
 void launch_coarse_batch(VecType vt, const CoarseArgs* args, const BItem* items, int32_t n_items, cudaStream_t st);
 
 }  // namespace amgsym

@@ -260,29 +260,53 @@ void launch_vec_batch(int op, VecType vt, int cpt, const UpdArgs* args, const BI
 
 // ---------------------------------------------------------------------------
 // Batched dense coarsest-level solve (FP64 arithmetic).  Item = a row range
-// [first_slot, row_end) of one problem's coarsest level.
+// [first_slot, row_end) of one problem's coarsest level, at most
+// kCoarseItemRows rows.  A thread sums kCoarseThreadRows rows of one column,
+// so each value of Y is converted to FP64 once for all of them.  The kernel is
+// bound by FP64 issue (2 lanes per clock per SM): an item is small enough
+// that a batch's rows cover the SMs (32-row items left nine SMs in ten idle
+// on 8 problems of 64 rows and 128 columns, 67 us a launch; that batch's solve
+// 327 -> 312 ms).
+constexpr int kCoarseThreadRows = 2;
 template <typename T>
 __global__ void __launch_bounds__(kBlock) coarse_batch_kernel(const CoarseArgs* __restrict__ args,
                                                              const BItem* __restrict__ items, int32_t n_items) {
+  constexpr int R = kCoarseThreadRows;
   for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
     const BItem bi = items[it];
     const CoarseArgs a = args[bi.arg];
     if (a.skip && *a.skip == 0) continue;
     const T* Y = static_cast<const T*>(a.Y);
     T* Z = static_cast<T*>(a.Z);
-    const int64_t r0 = bi.first_slot, r1 = bi.row_end;
-    const int64_t total = (r1 - r0) * a.C;
-    for (int64_t t = threadIdx.x; t < total; t += blockDim.x) {
-      const int64_t i = r0 + t / a.C, c = t % a.C;
-      const double* row = a.Ainv + i * a.n;
-      double acc0 = 0.0, acc1 = 0.0;
+    const int r0 = bi.first_slot, r1 = bi.row_end;
+    const int total = (r1 - r0 + R - 1) / R * a.C;
+    for (int t = threadIdx.x; t < total; t += blockDim.x) {
+      const int i = r0 + t / a.C * R, c = t % a.C;
+      const int nr = min(R, r1 - i);
+      // the rows past the range repeat the last one (their sums are not stored)
+      const double* row[R];
+#pragma unroll
+      for (int q = 0; q < R; ++q) row[q] = a.Ainv + (int64_t)(i + min(q, nr - 1)) * a.n;
+      double acc0[R], acc1[R];
+#pragma unroll
+      for (int q = 0; q < R; ++q) acc0[q] = acc1[q] = 0.0;
       int j = 0;
       for (; j + 1 < a.n; j += 2) {
-        acc0 = fma(row[j], (double)Y[(int64_t)j * a.C + c], acc0);
-        acc1 = fma(row[j + 1], (double)Y[(int64_t)(j + 1) * a.C + c], acc1);
+        const double y0 = (double)Y[(int64_t)j * a.C + c], y1 = (double)Y[(int64_t)(j + 1) * a.C + c];
+#pragma unroll
+        for (int q = 0; q < R; ++q) {
+          acc0[q] = fma(row[q][j], y0, acc0[q]);
+          acc1[q] = fma(row[q][j + 1], y1, acc1[q]);
+        }
       }
-      if (j < a.n) acc0 = fma(row[j], (double)Y[(int64_t)j * a.C + c], acc0);
-      Z[i * a.C + c] = (T)(acc0 + acc1);
+      if (j < a.n) {
+        const double y0 = (double)Y[(int64_t)j * a.C + c];
+#pragma unroll
+        for (int q = 0; q < R; ++q) acc0[q] = fma(row[q][j], y0, acc0[q]);
+      }
+#pragma unroll
+      for (int q = 0; q < R; ++q)
+        if (q < nr) Z[(int64_t)(i + q) * a.C + c] = (T)(acc0[q] + acc1[q]);
     }
   }
 }

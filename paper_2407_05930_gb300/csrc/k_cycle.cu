@@ -68,7 +68,7 @@ __device__ __forceinline__ void dense_phase(const CoarseArgs& c) {
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   coarse_rows_warp<XT>(c.n, c.C, c.Ainv, static_cast<const XT*>(c.Y), static_cast<XT*>(c.Z), warp, nwarps,
-                       [](const XT* p) { return ldv_cg<XT, 1>(p).v[0]; });
+                       [](const auto* p) { return __ldcg(p); });
 }
 
 // Diagonal smoother step, the arithmetic of the stand-alone jacobi kernel.
