@@ -146,11 +146,8 @@ static void resolve_tile(const SpmmArgs& a, VecType xt, VecType ot, int* cpt, in
     c = 1;
   if (xt == VEC_F64 || ot == VEC_F64) c = std::min(c, xt == VEC_F64 && ot == VEC_F64 ? 4 : 2);
   const int tpc = a.C / c;
-  int k = a.kl > 0 ? a.kl : 1;
-  if ((tpc & (tpc - 1)) || a.ndiag > 0) k = 1;
-  while (k > 1 && tpc * k > 32) k >>= 1;
   *cpt = c;
-  *kl = k;
+  *kl = a.ndiag > 0 ? 1 : clamp_lanes(tpc, a.kl > 0 ? a.kl : 1);
 }
 
 static void run_plan(const std::vector<BLaunch>& plan, cudaStream_t st);
@@ -183,7 +180,7 @@ static void add_spmm_core(Batch* B, std::vector<BLaunch>& plan, const std::vecto
       const int arg = (int)ga.size();
       ga.push_back(a);
       const int S = (a.C / L.cpt) * L.kl;
-      const int rows_pb = kBlock / S;
+      const int rows_pb = tile_rows_pb(a.C / L.cpt, L.kl);
       const int m = slots_per_item(a.rows, rows_pb, (int64_t)a.C * (xt == VEC_F64 ? 8 : 4));
       const int64_t slots = ((int64_t)a.rows + rows_pb - 1) / rows_pb;
       int32_t slot = 0;

@@ -208,6 +208,17 @@ struct SpmmArgs {
 
 // Launchers (k_spmm.cu).  mt: matrix values, xt: X/Z/W vectors, ot: Y.
 void launch_spmm(ValType mt, VecType xt, VecType ot, const SpmmArgs& a, cudaStream_t st);
+// Row slots of a 256-thread block when tpc column threads times kl entry lanes
+// serve a row (TileLayout in spmm_common.cuh).
+__host__ __device__ inline int tile_rows_pb(int tpc, int kl) {
+  const int S = tpc * kl;
+  return (kl > 1 && 32 % S) ? 8 * (32 / S) : 256 / S;
+}
+// Entry lanes of a row served by tpc column threads: a row slot stays in one warp.
+inline int clamp_lanes(int tpc, int kl) {
+  while (kl > 1 && tpc * kl > 32) kl >>= 1;
+  return kl;
+}
 // The (columns per thread, entry lanes) launch_spmm runs for these arguments.
 void spmm_resolved_tile(VecType xt, VecType ot, const SpmmArgs& a, int* cpt, int* kl);
 // Whether launch_spmm runs the halo-staged kernel for these arguments.

@@ -18,7 +18,7 @@
 namespace amgsym {
 
 template <typename MT, typename XT, typename OT, int CPT, int KL, bool HAS_DOT, bool HAS_IFACE, bool DIA>
-__global__ void __launch_bounds__(kBlock, 4)
+__global__ void __launch_bounds__(kBlock, (DIA && HAS_DOT) || sizeof(XT) == 8 ? 3 : 4)
     spmm_batch_kernel(const SpmmArgs* __restrict__ args, const BItem* __restrict__ items, int32_t n_items,
                       const BDot* __restrict__ dots) {
   using DT = typename AccOf<XT>::type;
@@ -31,17 +31,18 @@ __global__ void __launch_bounds__(kBlock, 4)
     if (threadIdx.x == 0) a = args[bi.arg];
     __syncthreads();
     if (a.skip && *a.skip == 0) continue;  // block-uniform
-    DT dpart[CPT];
+    constexpr int E = tile_cols<CPT, KL>();
+    DT dpart[E];
 #pragma unroll
-    for (int q = 0; q < CPT; ++q) dpart[q] = (DT)0;
+    for (int q = 0; q < E; ++q) dpart[q] = (DT)0;
     spmm_tile<MT, XT, OT, CPT, KL, HAS_DOT, HAS_IFACE, DIA>(a, bi.first_slot, 1, bi.row_end, dpart, false);
     if (HAS_DOT) {
       const TileLayout t = tile_layout<CPT, KL>(a.C);
-      double part[CPT];
+      double part[E];
 #pragma unroll
-      for (int q = 0; q < CPT; ++q) part[q] = (t.slot_ok && t.e == 0) ? (double)dpart[q] : 0.0;
+      for (int q = 0; q < E; ++q) part[q] = t.own ? (double)dpart[q] : 0.0;
       const BDot bd = dots[bi.arg];
-      block_dot2<CPT>(a.dot, part, t.c0, t.slot_ok && t.e == 0, t.g, t.rows_pb, t.S, a.C, sm, bi.slot, bd);
+      block_dot2<E>(a.dot, part, t.ec0, t.own, t.g, t.rows_pb, t.S, a.C, sm, bi.slot, bd);
     }
   }
 }

@@ -22,6 +22,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "coarse.cuh"
 #include "spmm_common.cuh"
@@ -105,17 +106,23 @@ __global__ void __launch_bounds__(kBlock, 2)
     } else if (ph.kind == CYCLE_JACOBI) {
       jacobi_phase<XT>(ph.j);
     } else {
-      DT dpart[CPT];
       const SpmmArgs& a = ph.a;
+      // no dot here: the partials are never touched
+      auto tile = [&](auto kl) {
+        constexpr int KL = decltype(kl)::value;
+        DT dpart[tile_cols<CPT, KL>()];
+        spmm_tile<MT, XT, XT, CPT, KL, false, false, false, true>(a, blockIdx.x, gridDim.x, a.rows, dpart);
+      };
       if (a.ndiag > 0) {
+        DT dpart[CPT];
         spmm_tile<MT, XT, XT, CPT, 1, false, false, true, true>(a, blockIdx.x, gridDim.x, a.rows, dpart);
       } else {
         switch (a.kl) {
-          case 1: spmm_tile<MT, XT, XT, CPT, 1, false, false, false, true>(a, blockIdx.x, gridDim.x, a.rows, dpart); break;
-          case 2: spmm_tile<MT, XT, XT, CPT, 2, false, false, false, true>(a, blockIdx.x, gridDim.x, a.rows, dpart); break;
-          case 4: spmm_tile<MT, XT, XT, CPT, 4, false, false, false, true>(a, blockIdx.x, gridDim.x, a.rows, dpart); break;
-          case 8: spmm_tile<MT, XT, XT, CPT, 8, false, false, false, true>(a, blockIdx.x, gridDim.x, a.rows, dpart); break;
-          default: spmm_tile<MT, XT, XT, CPT, 16, false, false, false, true>(a, blockIdx.x, gridDim.x, a.rows, dpart); break;
+          case 1: tile(std::integral_constant<int, 1>{}); break;
+          case 2: tile(std::integral_constant<int, 2>{}); break;
+          case 4: tile(std::integral_constant<int, 4>{}); break;
+          case 8: tile(std::integral_constant<int, 8>{}); break;
+          default: tile(std::integral_constant<int, 16>{}); break;
         }
       }
     }

@@ -38,12 +38,13 @@
 namespace amgsym {
 
 template <typename MT, typename XT, typename OT, int CPT, int KL, bool HAS_DOT, bool HAS_IFACE, bool DIA>
-__global__ void __launch_bounds__(kBlock, ((DIA && HAS_DOT) ? 3 : (DIA || CPT >= 8) ? 4 : (HAS_DOT || HAS_IFACE) ? 6 : 8)) spmm_kernel(SpmmArgs a) {
+__global__ void __launch_bounds__(kBlock, spmm_min_blocks<XT, CPT, HAS_DOT, HAS_IFACE, DIA>()) spmm_kernel(SpmmArgs a) {
   using DT = typename AccOf<XT>::type;
   if (a.skip && *a.skip == 0) return;  // uniform over the grid
-  DT dpart[CPT];
+  constexpr int E = tile_cols<CPT, KL>();
+  DT dpart[E];
 #pragma unroll
-  for (int q = 0; q < CPT; ++q) dpart[q] = (DT)0;
+  for (int q = 0; q < E; ++q) dpart[q] = (DT)0;
   // Grid-stride over row slots: a wave of blocks sweeps one contiguous window
   // of rows, so the far neighbours one block gathers were recently brought
   // into L2 by another.
@@ -51,11 +52,11 @@ __global__ void __launch_bounds__(kBlock, ((DIA && HAS_DOT) ? 3 : (DIA || CPT >=
   if (HAS_DOT) {
     const TileLayout t = tile_layout<CPT, KL>(a.C);
     extern __shared__ double sm[];
-    double part[CPT];
+    double part[E];
 #pragma unroll
-    for (int q = 0; q < CPT; ++q) part[q] = (t.slot_ok && t.e == 0) ? (double)dpart[q] : 0.0;
-    block_dot<CPT>(a.dot, part, t.c0, t.slot_ok && t.e == 0, t.g, t.rows_pb, t.S, a.C, sm, blockIdx.x,
-                   gridDim.x, a.dot.sc.partials, a.dot.sc.ticket);
+    for (int q = 0; q < E; ++q) part[q] = t.own ? (double)dpart[q] : 0.0;
+    block_dot<E>(a.dot, part, t.ec0, t.own, t.g, t.rows_pb, t.S, a.C, sm, blockIdx.x, gridDim.x, a.dot.sc.partials,
+                 a.dot.sc.ticket);
   }
 }
 
@@ -200,8 +201,12 @@ static size_t halo_smem_bytes(VecType xt, const SpmmArgs& a) {
 // The halo form pays off only with tiles enough to fill the GPU: a tile is
 // one block's serial stage-then-compute, so a small level with a few dozen
 // tiles runs faster as the CSR kernel's many short rows.
+// Its row slots are aligned to powers of two within a block.
 bool spmm_uses_halo(VecType xt, const SpmmArgs& a) {
-  return a.htiles >= 2 * num_sms() && a.hptr && a.ndiag <= 0 && a.dot.mode == DOT_NONE && !a.imask &&
+  int cpt = 0, kl = 0;
+  spmm_resolved_tile(xt, xt, a, &cpt, &kl);
+  const int tpc = a.C / cpt;
+  return (kl == 1 || (tpc & (tpc - 1)) == 0) && a.htiles >= 2 * num_sms() && a.hptr && a.ndiag <= 0 && a.dot.mode == DOT_NONE && !a.imask &&
          halo_smem_bytes(xt, a) <= (size_t)kHaloSmemLimit;
 }
 
@@ -231,7 +236,7 @@ static void launch_h(const SpmmArgs& a, cudaStream_t st) {
 template <typename MT, typename XT, typename OT, int CPT, int KL, bool DIA = false>
 static void launch_k(const SpmmArgs& a, cudaStream_t st) {
   const int TPC = a.C / CPT;
-  const int rows_pb = kBlock / (TPC * KL);
+  const int rows_pb = tile_rows_pb(TPC, KL);
   int64_t need = ((int64_t)a.rows + rows_pb - 1) / rows_pb;
   int grid = (int)std::min<int64_t>(need, (int64_t)max_grid_blocks());
   if (grid < 1) grid = 1;
@@ -284,10 +289,7 @@ static void launch_t(const SpmmArgs& a, cudaStream_t st) {
     return;
   }
   const int TPC = a.C / CPT;
-  // entry lanes: only with a power-of-two column-thread count, and S <= 32
-  int kl = a.kl > 0 ? a.kl : 1;
-  if (TPC & (TPC - 1)) kl = 1;
-  while (kl > 1 && TPC * kl > 32) kl >>= 1;
+  const int kl = clamp_lanes(TPC, a.kl > 0 ? a.kl : 1);
   if (spmm_uses_halo(sizeof(XT) == 8 ? VEC_F64 : VEC_F32, a)) {
     switch (kl) {
       case 1: launch_h<MT, XT, OT, CPT, 1>(a, st); break;
@@ -434,10 +436,7 @@ void spmm_resolved_tile(VecType xt, VecType ot, const SpmmArgs& a, int* cpt, int
     c = 1;
   int k = 1;
   if (a.ndiag <= 0) {
-    const int tpc = a.C / c;
-    k = a.kl > 0 ? a.kl : 1;
-    if (tpc & (tpc - 1)) k = 1;
-    while (k > 1 && tpc * k > 32) k >>= 1;
+    k = clamp_lanes(a.C / c, a.kl > 0 ? a.kl : 1);
   }
   *cpt = c;
   *kl = k;

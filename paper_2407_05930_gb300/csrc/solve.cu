@@ -692,10 +692,8 @@ Tile fixed_tile(const DevCsr& M, int32_t C, VecType xt) {
     t.cpt = V;
     t.kl = 16;
   }
-  if (C % t.cpt) t.cpt = (C % V == 0) ? V : 1;
-  const int tpc = C / t.cpt;
-  if (tpc & (tpc - 1)) t.kl = 1;
-  while (t.kl > 1 && tpc * t.kl > 32) t.kl >>= 1;
+  if (C % t.cpt) t.cpt = (C % V == 0) ? V : (C % 2 == 0) ? 2 : 1;
+  t.kl = clamp_lanes(C / t.cpt, t.kl);
   return t;
 }
 
@@ -840,7 +838,7 @@ void tune_tiles(const Ctx& c) {
       if (c.C % cpt) continue;
       const int tpc = c.C / cpt;
       for (int kl = 1; kl <= 16; kl *= 2) {
-        if (kl > 1 && ((tpc & (tpc - 1)) || tpc * kl > 32 || j.M->ndiag > 0)) break;
+        if (kl > 1 && (tpc * kl > 32 || j.M->ndiag > 0)) break;
         Ctx cc = c;
         const int var = j.dot ? 1 : 0;
         D->tiles[TileKey{j.M->idx, c.C, (int)j.mt, (int)c.vt, (int)c.vt, var}] = Tile{cpt, kl};
@@ -977,10 +975,7 @@ static void cycle_phase(const Ctx& c, std::vector<CyclePhase>& out, const DevCsr
   int cpt = 0, kl = 1;
   spmm_resolved_tile(c.vt, c.vt, ph.a, &cpt, &kl);
   // the kernel's own column split; entry lanes as the stand-alone launch
-  const int tpc = c.C / kcpt;
-  if (tpc & (tpc - 1)) kl = 1;
-  while (kl > 1 && tpc * kl > 32) kl >>= 1;
-  ph.a.kl = kl;
+  ph.a.kl = clamp_lanes(c.C / kcpt, kl);
   ph.a.cpt = kcpt;
   out.push_back(ph);
 }

@@ -153,6 +153,7 @@ __device__ __forceinline__ void dia_row(const SpmmArgs& a, int row, int c0, CT (
       }
 #pragma unroll
       for (int u = 0; u < UB; ++u) {
+        if (sizeof(CT) == 8 && d0 + u >= a.ndiag) continue;  // uniform
 #pragma unroll
         for (int q = 0; q < CPT; ++q) acc[q] = fma(m[u], (CT)x[u].v[q], acc[q]);
       }
@@ -163,7 +164,9 @@ __device__ __forceinline__ void dia_row(const SpmmArgs& a, int row, int c0, CT (
 // The CSR entries kb + e, kb + e + KL, ... < ke of one row, U per step,
 // predicated: all index/value loads first, then all gathers, so a row of up
 // to U * KL entries costs one round trip and a 7-point row (U = 4) two, with
-// every gather of a step in flight at once.
+// every gather of a step in flight at once.  FP64 sums skip the masked fmas: an
+// FP64 instruction takes 16 issue cycles whatever its lanes hold (2 lanes per
+// clock per SM), so a 19-entry row at KL = 4 costs 5 fmas per column, not 8.
 template <typename MT, typename XT, typename CT, int CPT, int KL, bool COH>
 __device__ __forceinline__ void csr_row(const SpmmArgs& a, int kb, int ke, int e, int c0, CT (&acc)[CPT]) {
   const MT* __restrict__ val = static_cast<const MT*>(a.val);
@@ -192,6 +195,7 @@ __device__ __forceinline__ void csr_row(const SpmmArgs& a, int kb, int ke, int e
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
+      if (sizeof(CT) == 8 && k + u * KL >= ke) continue;
 #pragma unroll
       for (int q = 0; q < CPT; ++q) acc[q] = fma(m[u], (CT)x[u].v[q], acc[q]);
     }
@@ -275,20 +279,24 @@ __device__ __forceinline__ void row_epilogue(const SpmmArgs& a, int row, int c0,
     // the epilogue operand as loaded early by the caller (use_zpre), else now;
     // passed by value so that it stays in registers
     const Vec<XT, CPT> zv = use_zpre ? zpre : ldx<XT, CPT, COH>(static_cast<const XT*>(a.Z) + (int64_t)row * C + c0);
+    // FP64: the factors +-1 of residuals and updates without their multiply
+    // (the same rounding: z - acc = fma(-1, acc, 1 * z))
+    if (sizeof(CT) == 8 && a.beta == 1.0 && a.alpha == -1.0) {
 #pragma unroll
-    for (int q = 0; q < CPT; ++q) {
-      const CT y = fma(alpha, acc[q], beta * (CT)zv.v[q]);
-      out.v[q] = (OT)y;
-      acc[q] = y;
-    }
-  } else {
+      for (int q = 0; q < CPT; ++q) acc[q] = (CT)zv.v[q] - acc[q];
+    } else if (sizeof(CT) == 8 && a.beta == 1.0) {
 #pragma unroll
-    for (int q = 0; q < CPT; ++q) {
-      const CT y = alpha * acc[q];
-      out.v[q] = (OT)y;
-      acc[q] = y;
+      for (int q = 0; q < CPT; ++q) acc[q] = fma(alpha, acc[q], (CT)zv.v[q]);
+    } else {
+#pragma unroll
+      for (int q = 0; q < CPT; ++q) acc[q] = fma(alpha, acc[q], beta * (CT)zv.v[q]);
     }
+  } else if (sizeof(CT) != 8 || a.alpha != 1.0) {
+#pragma unroll
+    for (int q = 0; q < CPT; ++q) acc[q] = alpha * acc[q];
   }
+#pragma unroll
+  for (int q = 0; q < CPT; ++q) out.v[q] = (OT)acc[q];
   if (a.jmode == 1) {
     // presmoothing of the next level from zero: Y2 = jd o Y, the arithmetic
     // of the stand-alone diagonal step (one product of the stored values)
@@ -319,17 +327,108 @@ __device__ __forceinline__ void row_epilogue(const SpmmArgs& a, int row, int c0,
   }
 }
 
+// Resident blocks per SM asked of the compiler.  FP64 with two vectors of
+// columns keeps 3 (80 registers: at 8 blocks the CSR kernels spilled 48 to 132
+// bytes a thread); its bound is FP64 issue, which a few warps saturate.
+template <typename XT, int CPT, bool HAS_DOT, bool HAS_IFACE, bool DIA>
+constexpr int spmm_min_blocks() {
+  return (DIA && HAS_DOT)                  ? 3
+         : sizeof(XT) == 8 && CPT >= 4     ? 3
+         : (DIA || CPT >= 8)               ? 4
+         : sizeof(XT) == 8 && CPT >= 2     ? 4
+         : (HAS_DOT || HAS_IFACE)          ? 6
+                                           : 8;
+}
+
+// The thread's place in the tile layout of one SpMM.  A row is served by
+// S = TPC * KL threads: TPC column threads (each owning CPT consecutive
+// columns, TPC = C / CPT) times KL entry lanes (lane e takes the row's entries
+// e, e + KL, ...).  When S divides a warp the row slots fill the block; else,
+// with KL > 1, each warp holds 32 / S slots and idles the rest of its lanes
+// (the lanes of a slot exchange by shuffles).
+//
+// The KL partial sums of a column combine by halving exchanges: the entry
+// lanes e and e ^ (KL / 2) swap half of their columns and add, then e and
+// e ^ (KL / 4), so a lane ends with E = max(1, CPT / KL) columns from ec0 and
+// runs the epilogue of those (dup: a lower lane holds them).  Against a full
+// exchange with the epilogue in lane 0 that is CPT - 1 instead of
+// CPT log2(KL) shuffles and adds, and an epilogue of E instead of CPT columns.
+// Each column's sum is the same tree.  Measured on whole solves to 1e-12 with
+// the skipped FP64 fmas: FP64 192^3 (C = 8, two solves) 302 -> 270 ms, FP64
+// ragged 87k rows at C = 12 (three column threads a row: one entry lane before)
+// 24.7 -> 18.4 ms, mixed 128^3 at C = 32 34.5 -> 32.0 ms.
+struct TileLayout {
+  int TPC, S, rows_pb, g, e, c0, ec0;
+  bool slot_ok, own;
+};
+
+template <int CPT, int KL>
+__host__ __device__ constexpr int tile_cols() {  // columns of a thread in the epilogue
+  return CPT / KL > 0 ? CPT / KL : 1;
+}
+
+template <int CPT, int KL>
+__device__ __forceinline__ TileLayout tile_layout(int C) {
+  TileLayout t;
+  t.TPC = C / CPT;
+  t.S = t.TPC * KL;
+  t.rows_pb = tile_rows_pb(t.TPC, KL);
+  int w;
+  if (KL > 1 && 32 % t.S) {
+    const int lane = threadIdx.x & 31, rpw = 32 / t.S, sl = lane / t.S;
+    t.g = (threadIdx.x >> 5) * rpw + sl;
+    t.slot_ok = sl < rpw;
+    w = lane - sl * t.S;
+  } else {
+    t.g = threadIdx.x / t.S;
+    t.slot_ok = t.g < t.rows_pb;
+    w = threadIdx.x - t.g * t.S;
+  }
+  t.e = KL > 1 ? w / t.TPC : 0;
+  t.c0 = (w - t.e * t.TPC) * CPT;
+  t.ec0 = t.c0;
+  t.own = t.slot_ok;
+#pragma unroll
+  for (int off = KL / 2, h = CPT / 2; off >= 1; off >>= 1, h >>= 1) {
+    if (t.e & off) {
+      if (h >= 1)
+        t.ec0 += h;
+      else
+        t.own = false;
+    }
+  }
+  return t;
+}
+
+// Combines the entry lanes' sums; the thread's columns are left in acc[0 .. E).
+template <int CPT, int KL, typename CT>
+__device__ __forceinline__ void combine_lanes(const TileLayout& t, CT (&acc)[CPT]) {
+#pragma unroll
+  for (int off = KL / 2, h = CPT / 2; off >= 1; off >>= 1, h >>= 1) {
+    const bool up = (t.e & off) != 0;
+    const int src = (threadIdx.x & 31) + (up ? -off : off) * t.TPC;  // (outside a slot: any lane)
+    if (h >= 1) {
+#pragma unroll
+      for (int q = 0; q < CPT / 2; ++q) {
+        if (q < h) {
+          const CT send = up ? acc[q] : acc[q + h];
+          const CT keep = up ? acc[q + h] : acc[q];
+          acc[q] = keep + __shfl_sync(0xffffffffu, send, src);
+        }
+      }
+    } else {
+      acc[0] += __shfl_sync(0xffffffffu, acc[0], src);
+    }
+  }
+}
+
 // Rows [first_slot * rows_pb + k * slot_step * rows_pb, ...) below row_end
-// of one SpMM, for the whole block; this thread's dot partial (entry lane 0
-// only) is added to dpart.  Thread layout: a row is served by S = TPC * KL
-// threads: TPC column threads (each owning CPT consecutive columns, TPC =
-// C / CPT) times KL entry lanes (lane e takes the row's entries e, e + KL,
-// ...).  The KL partial sums are combined with warp shuffles (S divides 32
-// when KL > 1), and entry lane 0 runs the epilogue.  KL > 1 keeps several
-// gathers of one row in flight (the ptr -> idx -> X latency chain) and spreads
-// the long rows of the coarse levels over many lanes.  DIA: the matrix is in
-// the diagonal-offset form (one lane per row, no row pointers).  COH: vector
-// operands are loaded through L2 only (written earlier in the same launch).
+// of one SpMM, for the whole block; this thread's dot partial (its epilogue
+// columns) is added to dpart.  KL > 1 keeps several gathers of one row in
+// flight (the ptr -> idx -> X latency chain) and spreads the long rows of the
+// coarse levels over many lanes.  DIA: the matrix is in the diagonal-offset
+// form (one lane per row, no row pointers).  COH: vector operands are loaded
+// through L2 only (written earlier in the same launch).
 //
 // Interface rows (HAS_IFACE) take a second pass: the main pass computes
 // every row but stores none of the flagged ones, so no row waits on the
@@ -343,10 +442,11 @@ __device__ __forceinline__ void row_epilogue(const SpmmArgs& a, int row, int c0,
 template <typename MT, typename XT, typename OT, int CPT, int KL, bool HAS_DOT, bool HAS_IFACE, bool DIA = false,
           bool COH = false>
 __device__ __forceinline__ void spmm_tile(const SpmmArgs& a, int first_slot, int slot_step, int row_end,
-                                          typename AccOf<XT>::type (&dpart)[CPT], bool whole = true) {
+                                          typename AccOf<XT>::type (&dpart)[tile_cols<CPT, KL>()], bool whole = true) {
   static_assert(!DIA || KL == 1, "the diagonal-offset form runs one entry lane per row");
   using CT = typename ComputeOf<MT, XT>::type;
   using DT = typename AccOf<XT>::type;  // per-thread dot partial type
+  constexpr int E = tile_cols<CPT, KL>();
   // Early epilogue-operand loads, issued with the row's matrix and X loads so
   // that the epilogue adds no dependent round trip: Z (beta != 0) in the CSR
   // variants launched at 6 blocks per SM, Z and the dot partner W in the
@@ -355,24 +455,16 @@ __device__ __forceinline__ void spmm_tile(const SpmmArgs& a, int first_slot, int
   constexpr bool DPF = HAS_DOT && DIA;
   constexpr bool PTR_PF = ZPF && !DIA;
   const int C = a.C;
-  const int TPC = C / CPT;
-  const int S = TPC * KL;
-  const int rows_pb = kBlock / S;
-  const int g = threadIdx.x / S;
-  const int w = threadIdx.x - g * S;
-  const int e = KL > 1 ? w / TPC : 0;
-  const int c0 = (w - e * TPC) * CPT;
-  const bool slot_ok = g < rows_pb;
+  const TileLayout t = tile_layout<CPT, KL>(C);
+  const int rows_pb = t.rows_pb, g = t.g, e = t.e, c0 = t.c0, ec0 = t.ec0;
+  const bool slot_ok = t.slot_ok;
   const XT* Z = static_cast<const XT*>(a.Z);
   const int32_t* __restrict__ ptr = a.ptr;
-  auto lanes = [&](CT (&acc)[CPT]) {
-    if (KL > 1) {
+  auto epilogue = [&](int row, CT (&acc)[CPT], const Vec<XT, E>& zpre, bool use_z, const Vec<XT, E>& wpre, bool use_w) {
+    CT out[E];
 #pragma unroll
-      for (int off = KL / 2; off >= 1; off >>= 1) {
-#pragma unroll
-        for (int q = 0; q < CPT; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], off * TPC);
-      }
-    }
+    for (int q = 0; q < E; ++q) out[q] = acc[q];
+    row_epilogue<XT, OT, CT, DT, E, HAS_DOT, COH>(a, row, ec0, out, zpre, use_z, wpre, use_w, dpart);
   };
 
   // The trip count is block-uniform (the shuffles need every lane of the warp).
@@ -391,10 +483,11 @@ __device__ __forceinline__ void spmm_tile(const SpmmArgs& a, int first_slot, int
   for (int base = first_slot * rows_pb; base < row_end; base += step_rows) {
     const int row = base + g;
     const bool live = slot_ok && row < row_end;
+    const bool own = t.own && live;  // this thread runs an epilogue
     CT acc[CPT];
 #pragma unroll
     for (int q = 0; q < CPT; ++q) acc[q] = (CT)0;
-    Vec<XT, CPT> zpre, wpre;
+    Vec<XT, E> zpre, wpre;
     int kb = kb_next, ke = ke_next;
     if (PTR_PF) {
       if (slot_ok && row + step_rows < row_end) {
@@ -409,20 +502,19 @@ __device__ __forceinline__ void spmm_tile(const SpmmArgs& a, int first_slot, int
     if (live) {
       // interface flag word and epilogue operand loaded with the row pointers,
       // off the critical path of the gathers
-      const uint32_t iface_word = (HAS_IFACE && e == 0) ? __ldg(a.imask + (row >> 5)) : 0u;
-      if ((ZPF || DPF) && e == 0 && a.beta != 0.0) zpre = ldx<XT, CPT, COH>(Z + (int64_t)row * C + c0);
-      if (DPF && e == 0 && a.dot.mode == DOT_WY)
-        wpre = ldx<XT, CPT, COH>(static_cast<const XT*>(a.dot.W) + (int64_t)row * C + c0);
+      const uint32_t iface_word = (HAS_IFACE && own) ? __ldg(a.imask + (row >> 5)) : 0u;
+      if ((ZPF || DPF) && own && a.beta != 0.0) zpre = ldx<XT, E, COH>(Z + (int64_t)row * C + ec0);
+      if (DPF && own && a.dot.mode == DOT_WY)
+        wpre = ldx<XT, E, COH>(static_cast<const XT*>(a.dot.W) + (int64_t)row * C + ec0);
       if (DIA)
         dia_row<MT, XT, CT, CPT, COH>(a, row, c0, acc);
       else
         csr_row<MT, XT, CT, CPT, KL, COH>(a, kb, ke, e, c0, acc);
       flagged = HAS_IFACE && (iface_word >> (row & 31)) & 1u;
     }
-    lanes(acc);
-    if (live && e == 0 && !flagged)
-      row_epilogue<XT, OT, CT, DT, CPT, HAS_DOT, COH>(a, row, c0, acc, zpre, (ZPF || DPF) && a.beta != 0.0, wpre,
-                                                      DPF && a.dot.mode == DOT_WY, dpart);
+    combine_lanes<CPT, KL, CT>(t, acc);
+    if (own && !flagged)
+      epilogue(row, acc, zpre, (ZPF || DPF) && a.beta != 0.0, wpre, DPF && a.dot.mode == DOT_WY);
   }
   if (HAS_IFACE) {
     // the flagged rows, with their couplings
@@ -444,32 +536,10 @@ __device__ __forceinline__ void spmm_tile(const SpmmArgs& a, int first_slot, int
         }
         if (e == 0) iface_row<XT, CT, CPT, COH>(a, f, c0, acc);
       }
-      lanes(acc);
-      if (live && e == 0)
-        row_epilogue<XT, OT, CT, DT, CPT, HAS_DOT, COH>(a, row, c0, acc, Vec<XT, CPT>{}, false, Vec<XT, CPT>{}, false,
-                                                        dpart);
+      combine_lanes<CPT, KL, CT>(t, acc);
+      if (t.own && live) epilogue(row, acc, Vec<XT, E>{}, false, Vec<XT, E>{}, false);
     }
   }
-}
-
-// The thread's place in the tile layout (see spmm_tile).
-struct TileLayout {
-  int S, rows_pb, g, e, c0;
-  bool slot_ok;
-};
-
-template <int CPT, int KL>
-__device__ __forceinline__ TileLayout tile_layout(int C) {
-  TileLayout t;
-  const int TPC = C / CPT;
-  t.S = TPC * KL;
-  t.rows_pb = kBlock / t.S;
-  t.g = threadIdx.x / t.S;
-  const int w = threadIdx.x - t.g * t.S;
-  t.e = KL > 1 ? w / TPC : 0;
-  t.c0 = (w - t.e * TPC) * CPT;
-  t.slot_ok = t.g < t.rows_pb;
-  return t;
 }
 
 }  // namespace amgsym
