@@ -6,6 +6,7 @@
 #include <atomic>
 #include <map>
 #include <mutex>
+#include <type_traits>
 
 #include "coarse.cuh"
 #include "device.h"
@@ -58,77 +59,154 @@ static int grid_for(int64_t work, int per_block) {
 // ---------------------------------------------------------------------------
 // Forward transform (Alg. 1, "Transform forward"; eq. "P_s" without the
 // 2^{-s/2} factor): gather the 2^s mirror images of every base cell through
-// perm, then s butterfly stages (a + b, a - b).  One thread per (rhs, l);
-// consecutive threads take consecutive l so the gathers of each copy and the
-// interleaved writes are coalesced.
+// perm, then s butterfly stages (a + b, a - b).  One thread per (rhs, l), the
+// right-hand side in blockIdx.y; consecutive threads take consecutive l, so
+// the gathers of each copy are coalesced.
+//
+// Bounds: the s 2^s FP64 adds per base cell first (24 at s = 3; 2 lanes per
+// clock per SM: 80 us at 256^3, against 49 us for the 335 MB at the copy
+// rate).  So nothing else runs on the FP64 pipe: the exact 2^-s of the way back
+// is an exponent subtraction, and a thread's 2^s values move as vectors of up
+// to 32 bytes (W values each, by the alignment of the reduced vector): as
+// single values every 8-byte access touched its own sector.
+// Measured at 256^3, s = 3, there and back: 248 -> 235 us.
+template <typename T, int W>
+struct alignas(sizeof(T) * W) TrVec {
+  T v[W];
+};
 
-template <int S, typename OT>
+// 32-byte vectors as one 256-bit access (sm_100 and later): whole sectors.
+template <typename T, int W>
+__device__ __forceinline__ void tr_store(T* p, const TrVec<T, W>& t) {
+  if constexpr (sizeof(T) == 8 && W == 4)
+    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(t.v[0]), "d"(t.v[1]), "d"(t.v[2]),
+                 "d"(t.v[3])
+                 : "memory");
+  else
+    *reinterpret_cast<TrVec<T, W>*>(p) = t;
+}
+template <typename T, int W>
+__device__ __forceinline__ TrVec<T, W> tr_load(const T* p) {
+  TrVec<T, W> t;
+  if constexpr (sizeof(T) == 8 && W == 4)
+    asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
+                 : "=d"(t.v[0]), "=d"(t.v[1]), "=d"(t.v[2]), "=d"(t.v[3])
+                 : "l"(p));
+  else
+    t = *reinterpret_cast<const TrVec<T, W>*>(p);
+  return t;
+}
+
+// v 2^-S: exponent arithmetic for normal results, else the product (zeros,
+// subnormals, infinities, NaN).
+template <int S>
+__device__ __forceinline__ double scale_down(double v) {
+  const int hi = __double2hiint(v);
+  const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;
+  if (e - (S + 1u) < 0x7ffu - (S + 1u)) return __hiloint2double(hi - (S << 20), __double2loint(v));
+  return v * (1.0 / (double)(1 << S));
+}
+
+template <int S>
+__device__ __forceinline__ void butterfly(double (&v)[1 << S]) {
+#pragma unroll
+  for (int st = 0; st < S; ++st) {
+#pragma unroll
+    for (int i = 0; i < (1 << S); ++i)
+      if (!(i & (1 << st))) {
+        const double a0 = v[i], a1 = v[i | (1 << st)];
+        v[i] = a0 + a1;
+        v[i | (1 << st)] = a0 - a1;
+      }
+  }
+}
+
+template <int S, int W, typename OT>
 __global__ void __launch_bounds__(kBlock) transform_fwd_kernel(const double* __restrict__ b, int32_t nrhs,
                                                                int64_t ld, const int32_t* __restrict__ perm,
                                                                int64_t n_b, OT* __restrict__ xhat) {
   constexpr int NB = 1 << S;
-  const int64_t total = n_b * nrhs;
   const int64_t C = (int64_t)nrhs * NB;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = t / n_b, l = t - r * n_b;
-    double v[NB];
+  for (int r = blockIdx.y; r < nrhs; r += gridDim.y) {
+    for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < n_b; l += (int64_t)gridDim.x * blockDim.x) {
+      double v[NB];
 #pragma unroll
-    for (int j = 0; j < NB; ++j) v[j] = __ldcs(b + r * ld + __ldcs(perm + j * n_b + l));
+      for (int j = 0; j < NB; ++j) v[j] = __ldcs(b + r * ld + __ldcs(perm + j * n_b + l));
+      butterfly<S>(v);
+      OT* o = xhat + l * C + r * NB;
 #pragma unroll
-    for (int st = 0; st < S; ++st) {
+      for (int i = 0; i < NB; i += W) {
+        TrVec<OT, W> t;
 #pragma unroll
-      for (int i = 0; i < NB; ++i)
-        if (!(i & (1 << st))) {
-          const double a0 = v[i], a1 = v[i | (1 << st)];
-          v[i] = a0 + a1;
-          v[i | (1 << st)] = a0 - a1;
-        }
+        for (int q = 0; q < W; ++q) t.v[q] = (OT)v[i + q];
+        tr_store<OT, W>(o + i, t);
+      }
     }
-    OT* o = xhat + l * C + r * NB;
-#pragma unroll
-    for (int i = 0; i < NB; ++i) o[i] = (OT)v[i];
   }
 }
 
-template <int S, typename IT>
+template <int S, int W, typename IT>
 __global__ void __launch_bounds__(kBlock) transform_bwd_kernel(const IT* __restrict__ xhat, int32_t nrhs,
                                                                const int32_t* __restrict__ perm, int64_t n_b,
                                                                double* __restrict__ x, int64_t ld) {
   constexpr int NB = 1 << S;
-  const int64_t total = n_b * nrhs;
   const int64_t C = (int64_t)nrhs * NB;
-  const double scale = 1.0 / (double)NB;  // 2^{-s}: exact
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = t / n_b, l = t - r * n_b;
-    double v[NB];
-    const IT* in = xhat + l * C + r * NB;
+  for (int r = blockIdx.y; r < nrhs; r += gridDim.y) {
+    for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < n_b; l += (int64_t)gridDim.x * blockDim.x) {
+      double v[NB];
+      int32_t to[NB];
+      const IT* in = xhat + l * C + r * NB;
 #pragma unroll
-    for (int i = 0; i < NB; ++i) v[i] = (double)in[i];
+      for (int i = 0; i < NB; i += W) {
+        const TrVec<IT, W> t = tr_load<IT, W>(in + i);
 #pragma unroll
-    for (int st = 0; st < S; ++st) {
+        for (int q = 0; q < W; ++q) v[i + q] = (double)t.v[q];
+      }
 #pragma unroll
-      for (int i = 0; i < NB; ++i)
-        if (!(i & (1 << st))) {
-          const double a0 = v[i], a1 = v[i | (1 << st)];
-          v[i] = a0 + a1;
-          v[i | (1 << st)] = a0 - a1;
-        }
+      for (int j = 0; j < NB; ++j) to[j] = __ldcs(perm + j * n_b + l);
+      butterfly<S>(v);
+#pragma unroll
+      for (int j = 0; j < NB; ++j) __stcs(x + r * ld + to[j], scale_down<S>(v[j]));
     }
-#pragma unroll
-    for (int j = 0; j < NB; ++j) __stcs(x + r * ld + __ldcs(perm + j * n_b + l), v[j] * scale);
   }
+}
+
+// Values per vector: the widest of 32 bytes or less that a thread's 2^S values
+// fill and the reduced vector's address allows.
+template <int S, typename T, typename F>
+static void transform_width(const void* xhat, F&& run) {
+  constexpr int NB = 1 << S, W4 = 32 / (int)sizeof(T), W2 = 16 / (int)sizeof(T);
+  constexpr int WA = NB < W4 ? NB : W4, WB = NB < W2 ? NB : W2;
+  const uintptr_t p = (uintptr_t)xhat;
+  if (p % (WA * sizeof(T)) == 0)
+    run(std::integral_constant<int, WA>{});
+  else if (p % (WB * sizeof(T)) == 0)
+    run(std::integral_constant<int, WB>{});
+  else
+    run(std::integral_constant<int, 1>{});
+}
+
+static dim3 transform_grid(int64_t n_b, int32_t nrhs) {
+  const int64_t gx = std::max<int64_t>(1, std::min<int64_t>((n_b + kBlock - 1) / kBlock, max_grid_blocks()));
+  return dim3((unsigned)gx, (unsigned)std::max<int64_t>(1, std::min<int64_t>(nrhs, (max_grid_blocks() + gx - 1) / gx)));
 }
 
 template <typename OT>
 static void fwd_dispatch(const double* b, int32_t nrhs, int64_t ld, const int32_t* perm, int64_t n_b, int32_t s,
                          OT* xhat, cudaStream_t st) {
-  const int g = grid_for(n_b * nrhs, kBlock);
+  const dim3 g = transform_grid(n_b, nrhs);
+  auto go = [&](auto sc) {
+    constexpr int S = decltype(sc)::value;
+    transform_width<S, OT>(xhat, [&](auto w) {
+      transform_fwd_kernel<S, decltype(w)::value, OT><<<g, kBlock, 0, st>>>(b, nrhs, ld, perm, n_b, xhat);
+    });
+  };
   switch (s) {
-    case 0: transform_fwd_kernel<0, OT><<<g, kBlock, 0, st>>>(b, nrhs, ld, perm, n_b, xhat); break;
-    case 1: transform_fwd_kernel<1, OT><<<g, kBlock, 0, st>>>(b, nrhs, ld, perm, n_b, xhat); break;
-    case 2: transform_fwd_kernel<2, OT><<<g, kBlock, 0, st>>>(b, nrhs, ld, perm, n_b, xhat); break;
-    case 3: transform_fwd_kernel<3, OT><<<g, kBlock, 0, st>>>(b, nrhs, ld, perm, n_b, xhat); break;
-    case 4: transform_fwd_kernel<4, OT><<<g, kBlock, 0, st>>>(b, nrhs, ld, perm, n_b, xhat); break;
+    case 0: go(std::integral_constant<int, 0>{}); break;
+    case 1: go(std::integral_constant<int, 1>{}); break;
+    case 2: go(std::integral_constant<int, 2>{}); break;
+    case 3: go(std::integral_constant<int, 3>{}); break;
+    case 4: go(std::integral_constant<int, 4>{}); break;
     default: fail(AMGSYM_ERR_ARG, "the device transform supports s <= 4");
   }
 }
@@ -145,13 +223,19 @@ void launch_transform_fwd(const double* b, int32_t nrhs, int64_t ld, const int32
 template <typename IT>
 static void bwd_dispatch(const IT* xhat, int32_t nrhs, const int32_t* perm, int64_t n_b, int32_t s, double* x,
                          int64_t ld, cudaStream_t st) {
-  const int g = grid_for(n_b * nrhs, kBlock);
+  const dim3 g = transform_grid(n_b, nrhs);
+  auto go = [&](auto sc) {
+    constexpr int S = decltype(sc)::value;
+    transform_width<S, IT>(xhat, [&](auto w) {
+      transform_bwd_kernel<S, decltype(w)::value, IT><<<g, kBlock, 0, st>>>(xhat, nrhs, perm, n_b, x, ld);
+    });
+  };
   switch (s) {
-    case 0: transform_bwd_kernel<0, IT><<<g, kBlock, 0, st>>>(xhat, nrhs, perm, n_b, x, ld); break;
-    case 1: transform_bwd_kernel<1, IT><<<g, kBlock, 0, st>>>(xhat, nrhs, perm, n_b, x, ld); break;
-    case 2: transform_bwd_kernel<2, IT><<<g, kBlock, 0, st>>>(xhat, nrhs, perm, n_b, x, ld); break;
-    case 3: transform_bwd_kernel<3, IT><<<g, kBlock, 0, st>>>(xhat, nrhs, perm, n_b, x, ld); break;
-    case 4: transform_bwd_kernel<4, IT><<<g, kBlock, 0, st>>>(xhat, nrhs, perm, n_b, x, ld); break;
+    case 0: go(std::integral_constant<int, 0>{}); break;
+    case 1: go(std::integral_constant<int, 1>{}); break;
+    case 2: go(std::integral_constant<int, 2>{}); break;
+    case 3: go(std::integral_constant<int, 3>{}); break;
+    case 4: go(std::integral_constant<int, 4>{}); break;
     default: fail(AMGSYM_ERR_ARG, "the device transform supports s <= 4");
   }
 }
