@@ -21,6 +21,7 @@ template <typename MT, typename XT, typename OT, int CPT, int KL, bool HAS_DOT, 
 __global__ void __launch_bounds__(kBlock, (DIA && HAS_DOT) || sizeof(XT) == 8 ? 3 : 4)
     spmm_batch_kernel(const SpmmArgs* __restrict__ args, const BItem* __restrict__ items, int32_t n_items,
                       const BDot* __restrict__ dots) {
+  pdl_wait();
   using DT = typename AccOf<XT>::type;
   __shared__ __align__(16) unsigned char sa_raw[sizeof(SpmmArgs)];
   SpmmArgs& a = *reinterpret_cast<SpmmArgs*>(sa_raw);
@@ -52,7 +53,7 @@ static void spmm_batch_k(bool dot, bool iface, const SpmmArgs* args, const BItem
                          const BDot* dots, size_t smem, cudaStream_t st) {
   auto run = [&](auto kern) {
     const int g = std::max(1, std::min<int>(n_items, resident_grid((const void*)kern, smem)));
-    kern<<<g, kBlock, smem, st>>>(args, items, n_items, dots);
+    launch_pdl(kern, g, kBlock, smem, st, args, items, n_items, dots);
   };
   if (dot) {
     if (iface)
@@ -126,6 +127,7 @@ template <typename T, int CPT, int OP>
 __global__ void __launch_bounds__(kBlock) vec_batch_kernel(const UpdArgs* __restrict__ args,
                                                           const BItem* __restrict__ items, int32_t n_items,
                                                           const BDot* __restrict__ dots) {
+  pdl_wait();
   using DT = typename AccOf<T>::type;
   using V = VecB<T, CPT>;
   __shared__ __align__(16) unsigned char ua_raw[sizeof(UpdArgs)];
@@ -228,7 +230,7 @@ static void vec_batch_c(int op, const UpdArgs* args, const BItem* items, int32_t
                         size_t smem, cudaStream_t st) {
   auto run = [&](auto kern) {
     const int g = std::max(1, std::min<int>(n_items, resident_grid((const void*)kern, smem)));
-    kern<<<g, kBlock, smem, st>>>(args, items, n_items, dots);
+    launch_pdl(kern, g, kBlock, smem, st, args, items, n_items, dots);
   };
   if (op == BOP_UPDATE1)
     run(vec_batch_kernel<T, CPT, BOP_UPDATE1>);
@@ -272,6 +274,7 @@ constexpr int kCoarseThreadRows = 2;
 template <typename T>
 __global__ void __launch_bounds__(kBlock) coarse_batch_kernel(const CoarseArgs* __restrict__ args,
                                                              const BItem* __restrict__ items, int32_t n_items) {
+  pdl_wait();
   constexpr int R = kCoarseThreadRows;
   for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
     const BItem bi = items[it];
@@ -317,9 +320,9 @@ void launch_coarse_batch(VecType vt, const CoarseArgs* args, const BItem* items,
   count_launch();
   const int g = std::min<int>(n_items, max_grid_blocks());
   if (vt == VEC_F64)
-    coarse_batch_kernel<double><<<g, kBlock, 0, st>>>(args, items, n_items);
+    launch_pdl(coarse_batch_kernel<double>, g, kBlock, 0, st, args, items, n_items);
   else
-    coarse_batch_kernel<float><<<g, kBlock, 0, st>>>(args, items, n_items);
+    launch_pdl(coarse_batch_kernel<float>, g, kBlock, 0, st, args, items, n_items);
 }
 
 }  // namespace amgsym

@@ -28,6 +28,7 @@ constexpr int kJChunk = 8;  // vectors of a set per pass over W
 __global__ void __launch_bounds__(kBlock) mdot_partial_kernel(const double* __restrict__ V, int64_t vstride,
                                                               int32_t Cv, int32_t J, const double* __restrict__ W,
                                                               int64_t rows, int32_t C, double* __restrict__ part) {
+  pdl_wait();
   __shared__ double sm[kJChunk * kBlock];  // [line][u][column]
   const int rpb = kBlock / C;  // rows per block step
   const int col = threadIdx.x % C, rl = threadIdx.x / C;
@@ -84,6 +85,7 @@ __global__ void __launch_bounds__(kBlock) mdot_partial_kernel(const double* __re
 constexpr int kFinalCols = 8;
 __global__ void __launch_bounds__(kBlock) mdot_final_kernel(const double* __restrict__ part, int32_t nblk, int32_t n,
                                                             double* __restrict__ H) {
+  pdl_wait();
   __shared__ double sm[kBlock];
   constexpr int kSlices = kBlock / kFinalCols;
   const int t = blockIdx.x * kFinalCols + threadIdx.x % kFinalCols;
@@ -111,6 +113,7 @@ __global__ void __launch_bounds__(kBlock) mdot_final_kernel(const double* __rest
 __global__ void __launch_bounds__(kBlock) maxpy_kernel(const double* __restrict__ V, int64_t vstride, int32_t Cv,
                                                        int32_t J, const double* __restrict__ H, double sign,
                                                        double* __restrict__ W, int64_t rows, int32_t C) {
+  pdl_wait();
   const int64_t total = rows * C;
   for (int64_t e = blockIdx.x * (int64_t)kBlock + threadIdx.x; e < total; e += (int64_t)gridDim.x * kBlock) {
     const int64_t row = e / C;
@@ -125,6 +128,7 @@ __global__ void __launch_bounds__(kBlock) maxpy_kernel(const double* __restrict_
 // Out[row][c] = W[row][c] * s[c].
 __global__ void __launch_bounds__(kBlock) colscale_kernel(const double* __restrict__ W, const double* __restrict__ s,
                                                           double* __restrict__ out, int64_t rows, int32_t C) {
+  pdl_wait();
   const int64_t total = rows * C;
   for (int64_t e = blockIdx.x * (int64_t)kBlock + threadIdx.x; e < total; e += (int64_t)gridDim.x * kBlock)
     out[e] = W[e] * s[e % C];
@@ -146,20 +150,20 @@ void launch_mdot(const double* V, int64_t vstride, int32_t Cv, int32_t J, const 
   if (J <= 0) return;
   const int g = mdot_blocks(rows, C);
   count_launch(2);
-  mdot_partial_kernel<<<g, kBlock, 0, st>>>(V, vstride, Cv, J, W, rows, C, part);
-  mdot_final_kernel<<<(J * C + kFinalCols - 1) / kFinalCols, kBlock, 0, st>>>(part, g, J * C, H);
+  launch_pdl(mdot_partial_kernel, g, kBlock, 0, st, V, vstride, Cv, J, W, rows, C, part);
+  launch_pdl(mdot_final_kernel, (J * C + kFinalCols - 1) / kFinalCols, kBlock, 0, st, part, g, J * C, H);
 }
 
 void launch_maxpy(const double* V, int64_t vstride, int32_t Cv, int32_t J, const double* H, double sign, double* W,
                   int64_t rows, int32_t C, cudaStream_t st) {
   if (J <= 0) return;
   count_launch();
-  maxpy_kernel<<<grid_elems(rows * C), kBlock, 0, st>>>(V, vstride, Cv, J, H, sign, W, rows, C);
+  launch_pdl(maxpy_kernel, grid_elems(rows * C), kBlock, 0, st, V, vstride, Cv, J, H, sign, W, rows, C);
 }
 
 void launch_colscale(const double* W, const double* s, double* out, int64_t rows, int32_t C, cudaStream_t st) {
   count_launch();
-  colscale_kernel<<<grid_elems(rows * C), kBlock, 0, st>>>(W, s, out, rows, C);
+  launch_pdl(colscale_kernel, grid_elems(rows * C), kBlock, 0, st, W, s, out, rows, C);
 }
 
 }  // namespace amgsym

@@ -125,6 +125,7 @@ template <int S, int W, typename OT>
 __global__ void __launch_bounds__(kBlock) transform_fwd_kernel(const double* __restrict__ b, int32_t nrhs,
                                                                int64_t ld, const int32_t* __restrict__ perm,
                                                                int64_t n_b, OT* __restrict__ xhat) {
+  pdl_wait();
   constexpr int NB = 1 << S;
   const int64_t C = (int64_t)nrhs * NB;
   for (int r = blockIdx.y; r < nrhs; r += gridDim.y) {
@@ -149,6 +150,7 @@ template <int S, int W, typename IT>
 __global__ void __launch_bounds__(kBlock) transform_bwd_kernel(const IT* __restrict__ xhat, int32_t nrhs,
                                                                const int32_t* __restrict__ perm, int64_t n_b,
                                                                double* __restrict__ x, int64_t ld) {
+  pdl_wait();
   constexpr int NB = 1 << S;
   const int64_t C = (int64_t)nrhs * NB;
   for (int r = blockIdx.y; r < nrhs; r += gridDim.y) {
@@ -198,7 +200,7 @@ static void fwd_dispatch(const double* b, int32_t nrhs, int64_t ld, const int32_
   auto go = [&](auto sc) {
     constexpr int S = decltype(sc)::value;
     transform_width<S, OT>(xhat, [&](auto w) {
-      transform_fwd_kernel<S, decltype(w)::value, OT><<<g, kBlock, 0, st>>>(b, nrhs, ld, perm, n_b, xhat);
+      launch_pdl(transform_fwd_kernel<S, decltype(w)::value, OT>, g, kBlock, 0, st, b, nrhs, ld, perm, n_b, xhat);
     });
   };
   switch (s) {
@@ -227,7 +229,7 @@ static void bwd_dispatch(const IT* xhat, int32_t nrhs, const int32_t* perm, int6
   auto go = [&](auto sc) {
     constexpr int S = decltype(sc)::value;
     transform_width<S, IT>(xhat, [&](auto w) {
-      transform_bwd_kernel<S, decltype(w)::value, IT><<<g, kBlock, 0, st>>>(xhat, nrhs, perm, n_b, x, ld);
+      launch_pdl(transform_bwd_kernel<S, decltype(w)::value, IT>, g, kBlock, 0, st, xhat, nrhs, perm, n_b, x, ld);
     });
   };
   switch (s) {
@@ -273,6 +275,7 @@ __global__ void __launch_bounds__(kBlock) cg_update1_kernel(int64_t rows, int32_
                                                             T* __restrict__ r, const T* __restrict__ p,
                                                             const T* __restrict__ q, DotArgs dot,
                                                             const int32_t* skip) {
+  pdl_wait();
   using DT = typename DotAcc<T>::type;
   using V = VecM<T, CPT>;
   if (skip && *skip == 0) return;
@@ -322,7 +325,7 @@ static void update1_c(int64_t rows, int32_t C, void* x, void* r, const void* p, 
   int g = grid_for(rows, rows_pb > 0 ? rows_pb : 1);
   g = std::min(g, resident_grid((const void*)cg_update1_kernel<T, CPT, true>, smem));
   if ((int64_t)g * C > dot.sc.partial_cap) g = (int)(dot.sc.partial_cap / C);
-  cg_update1_kernel<T, CPT, true><<<g, kBlock, smem, st>>>(rows, C, static_cast<T*>(x), static_cast<T*>(r),
+  launch_pdl(cg_update1_kernel<T, CPT, true>, g, kBlock, smem, st, rows, C, static_cast<T*>(x), static_cast<T*>(r),
                                                         static_cast<const T*>(p), static_cast<const T*>(q), dot, skip);
 }
 
@@ -352,6 +355,7 @@ template <typename T, int CPT>
 __global__ void __launch_bounds__(kBlock) cg_update2_kernel(int64_t rows, int32_t C, T* __restrict__ p,
                                                             const T* __restrict__ z, const double* __restrict__ beta,
                                                             const int32_t* skip) {
+  pdl_wait();
   using V = VecM<T, CPT>;
   if (skip && *skip == 0) return;
   const int TPR = C / CPT;
@@ -377,7 +381,7 @@ static void update2_c(int64_t rows, int32_t C, void* p, const void* z, const dou
                       const int32_t* skip) {
   const int rows_pb = kBlock / (C / CPT);
   const int g = grid_for(rows, rows_pb > 0 ? rows_pb : 1);
-  cg_update2_kernel<T, CPT><<<g, kBlock, 0, st>>>(rows, C, static_cast<T*>(p), static_cast<const T*>(z), beta, skip);
+  launch_pdl(cg_update2_kernel<T, CPT>, g, kBlock, 0, st, rows, C, static_cast<T*>(p), static_cast<const T*>(z), beta, skip);
 }
 
 template <typename T>
@@ -407,6 +411,7 @@ template <typename T, int V>
 __global__ void __launch_bounds__(kBlock) jacobi_kernel(int64_t rows, int32_t C, const T* __restrict__ jd,
                                                         const T* __restrict__ src, T* z, int accumulate,
                                                         const int32_t* skip) {
+  pdl_wait();
   if (skip && *skip == 0) return;
   const int64_t slices = (int64_t)rows * (C / V);
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < slices; t += (int64_t)gridDim.x * blockDim.x) {
@@ -429,22 +434,23 @@ void launch_jacobi(VecType vt, int64_t rows, int32_t C, const void* jd, const vo
     const double* s = static_cast<const double*>(src);
     double* d = static_cast<double*>(z);
     if (C % 2 == 0)
-      jacobi_kernel<double, 2><<<grid_for(rows * (C / 2), kBlock), kBlock, 0, st>>>(rows, C, j, s, d, accumulate, skip);
+      launch_pdl(jacobi_kernel<double, 2>, grid_for(rows * (C / 2), kBlock), kBlock, 0, st, rows, C, j, s, d, accumulate, skip);
     else
-      jacobi_kernel<double, 1><<<grid_for(rows * C, kBlock), kBlock, 0, st>>>(rows, C, j, s, d, accumulate, skip);
+      launch_pdl(jacobi_kernel<double, 1>, grid_for(rows * C, kBlock), kBlock, 0, st, rows, C, j, s, d, accumulate, skip);
   } else {
     const float* j = static_cast<const float*>(jd);
     const float* s = static_cast<const float*>(src);
     float* d = static_cast<float*>(z);
     if (C % 4 == 0)
-      jacobi_kernel<float, 4><<<grid_for(rows * (C / 4), kBlock), kBlock, 0, st>>>(rows, C, j, s, d, accumulate, skip);
+      launch_pdl(jacobi_kernel<float, 4>, grid_for(rows * (C / 4), kBlock), kBlock, 0, st, rows, C, j, s, d, accumulate, skip);
     else
-      jacobi_kernel<float, 1><<<grid_for(rows * C, kBlock), kBlock, 0, st>>>(rows, C, j, s, d, accumulate, skip);
+      launch_pdl(jacobi_kernel<float, 1>, grid_for(rows * C, kBlock), kBlock, 0, st, rows, C, j, s, d, accumulate, skip);
   }
 }
 
 template <typename T>
 __global__ void add_to_f64_kernel(int64_t count, double* __restrict__ y, const T* __restrict__ x) {
+  pdl_wait();
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x)
     y[e] += (double)x[e];
 }
@@ -453,13 +459,14 @@ void launch_add_to_f64(VecType xt, int64_t count, double* y, const void* x, cuda
   count_launch();
   const int g = grid_for(count, kBlock);
   if (xt == VEC_F64)
-    add_to_f64_kernel<double><<<g, kBlock, 0, st>>>(count, y, static_cast<const double*>(x));
+    launch_pdl(add_to_f64_kernel<double>, g, kBlock, 0, st, count, y, static_cast<const double*>(x));
   else
-    add_to_f64_kernel<float><<<g, kBlock, 0, st>>>(count, y, static_cast<const float*>(x));
+    launch_pdl(add_to_f64_kernel<float>, g, kBlock, 0, st, count, y, static_cast<const float*>(x));
 }
 
 template <typename T>
 __global__ void copy_kernel(int64_t count, T* __restrict__ d, const T* __restrict__ s) {
+  pdl_wait();
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x)
     d[e] = s[e];
 }
@@ -468,13 +475,14 @@ void launch_copy(VecType vt, int64_t count, void* dst, const void* src, cudaStre
   count_launch();
   const int g = grid_for(count, kBlock);
   if (vt == VEC_F64)
-    copy_kernel<double><<<g, kBlock, 0, st>>>(count, static_cast<double*>(dst), static_cast<const double*>(src));
+    launch_pdl(copy_kernel<double>, g, kBlock, 0, st, count, static_cast<double*>(dst), static_cast<const double*>(src));
   else
-    copy_kernel<float><<<g, kBlock, 0, st>>>(count, static_cast<float*>(dst), static_cast<const float*>(src));
+    launch_pdl(copy_kernel<float>, g, kBlock, 0, st, count, static_cast<float*>(dst), static_cast<const float*>(src));
 }
 
 template <typename T>
 __global__ void zero_kernel(int64_t count, T* __restrict__ d) {
+  pdl_wait();
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x)
     d[e] = (T)0;
 }
@@ -483,9 +491,9 @@ void launch_zero(VecType vt, int64_t count, void* dst, cudaStream_t st) {
   count_launch();
   const int g = grid_for(count, kBlock);
   if (vt == VEC_F64)
-    zero_kernel<double><<<g, kBlock, 0, st>>>(count, static_cast<double*>(dst));
+    launch_pdl(zero_kernel<double>, g, kBlock, 0, st, count, static_cast<double*>(dst));
   else
-    zero_kernel<float><<<g, kBlock, 0, st>>>(count, static_cast<float*>(dst));
+    launch_pdl(zero_kernel<float>, g, kBlock, 0, st, count, static_cast<float*>(dst));
 }
 
 // Per-column dots of two [rows][C] vectors.  A thread owns CPT consecutive
@@ -497,6 +505,7 @@ void launch_zero(VecType vt, int64_t count, void* dst, cudaStream_t st) {
 template <typename T, int CPT>
 __global__ void __launch_bounds__(kBlock) dot_kernel(int64_t rows, int32_t C, const T* __restrict__ a,
                                                      const T* __restrict__ b, DotArgs dot, const int32_t* skip) {
+  pdl_wait();
   using DT = typename DotAcc<T>::type;
   using V = VecM<T, CPT>;
   if (skip && *skip == 0) return;
@@ -530,7 +539,7 @@ static void dot_c(int64_t rows, int32_t C, const void* a, const void* b, const D
   int g = grid_for(rows, rows_pb > 0 ? rows_pb : 1);
   if ((int64_t)g * C > dot.sc.partial_cap) g = (int)(dot.sc.partial_cap / C);
   const size_t smem = sizeof(double) * (size_t)dot_smem_doubles(TPR, rows_pb, C);
-  dot_kernel<T, CPT><<<g, kBlock, smem, st>>>(rows, C, static_cast<const T*>(a), static_cast<const T*>(b), dot, skip);
+  launch_pdl(dot_kernel<T, CPT>, g, kBlock, smem, st, rows, C, static_cast<const T*>(a), static_cast<const T*>(b), dot, skip);
 }
 
 void launch_dot(VecType vt, int64_t rows, int32_t C, const void* a, const void* b, const DotArgs& dot,
@@ -563,6 +572,7 @@ template <typename T>
 __global__ void __launch_bounds__(kCoarseBlock) coarse_kernel(int32_t n, int32_t C, const double* __restrict__ Ainv,
                                                         const T* __restrict__ Y, T* __restrict__ Z,
                                                         const int32_t* skip) {
+  pdl_wait();
   if (skip && *skip == 0) return;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -575,9 +585,9 @@ void launch_coarse_solve(VecType vt, int32_t n, int32_t C, const double* Ainv, c
   constexpr int wpb = kCoarseBlock / 32;
   const int g = (int)std::max<int64_t>(1, std::min<int64_t>((coarse_units(n, C) + wpb - 1) / wpb, 16 * num_sms()));
   if (vt == VEC_F64)
-    coarse_kernel<double><<<g, kCoarseBlock, 0, st>>>(n, C, Ainv, static_cast<const double*>(Y), static_cast<double*>(Z), skip);
+    launch_pdl(coarse_kernel<double>, g, kCoarseBlock, 0, st, n, C, Ainv, static_cast<const double*>(Y), static_cast<double*>(Z), skip);
   else
-    coarse_kernel<float><<<g, kCoarseBlock, 0, st>>>(n, C, Ainv, static_cast<const float*>(Y), static_cast<float*>(Z), skip);
+    launch_pdl(coarse_kernel<float>, g, kCoarseBlock, 0, st, n, C, Ainv, static_cast<const float*>(Y), static_cast<float*>(Z), skip);
 }
 
 // ---------------------------------------------------------------------------
@@ -590,6 +600,7 @@ void launch_coarse_solve(VecType vt, int32_t n, int32_t C, const double* Ainv, c
 __global__ void __launch_bounds__(kBlock) block0_partial_kernel(const double* __restrict__ X, int64_t rows,
                                                                 int32_t C, int32_t nb, int32_t nrhs,
                                                                 double* __restrict__ part) {
+  pdl_wait();
   __shared__ double sm[kBlock];
   for (int32_t r = 0; r < nrhs; ++r) {
     double acc = 0.0;
@@ -607,6 +618,7 @@ __global__ void __launch_bounds__(kBlock) block0_partial_kernel(const double* __
 }
 
 __global__ void block0_mean_kernel(double* part, int32_t nblocks, int32_t nrhs, int64_t rows) {
+  pdl_wait();
   for (int32_t r = threadIdx.x; r < nrhs; r += blockDim.x) {
     double acc = 0.0;
     for (int32_t g = 0; g < nblocks; ++g) acc += part[(int64_t)g * nrhs + r];
@@ -616,6 +628,7 @@ __global__ void block0_mean_kernel(double* part, int32_t nblocks, int32_t nrhs, 
 
 __global__ void __launch_bounds__(kBlock) block0_sub_kernel(double* __restrict__ X, int64_t rows, int32_t C,
                                                             int32_t nb, int32_t nrhs, const double* __restrict__ mean) {
+  pdl_wait();
   const int64_t total = rows * nrhs;
   for (int64_t t = blockIdx.x * (int64_t)kBlock + threadIdx.x; t < total; t += (int64_t)gridDim.x * kBlock) {
     const int64_t i = t / nrhs;
@@ -630,9 +643,9 @@ void launch_sub_block0_mean(double* X, int64_t rows, int32_t nrhs, int32_t nb, d
   int64_t g = std::min<int64_t>(max_grid_blocks(), (rows + kBlock - 1) / kBlock);
   g = std::max<int64_t>(1, std::min<int64_t>(g, scratch_cap / nrhs - 1));
   count_launch(3);
-  block0_partial_kernel<<<(int)g, kBlock, 0, st>>>(X, rows, C, nb, nrhs, scratch);
-  block0_mean_kernel<<<1, 256, 0, st>>>(scratch, (int32_t)g, nrhs, rows);
-  block0_sub_kernel<<<grid_for(rows * nrhs, kBlock), kBlock, 0, st>>>(X, rows, C, nb, nrhs, scratch + g * nrhs);
+  launch_pdl(block0_partial_kernel, (int)g, kBlock, 0, st, X, rows, C, nb, nrhs, scratch);
+  launch_pdl(block0_mean_kernel, 1, 256, 0, st, scratch, (int32_t)g, nrhs, rows);
+  launch_pdl(block0_sub_kernel, grid_for(rows * nrhs, kBlock), kBlock, 0, st, X, rows, C, nb, nrhs, scratch + g * nrhs);
 }
 
 // ---------------------------------------------------------------------------
@@ -649,6 +662,7 @@ template <typename T, int NB>
 __global__ void __launch_bounds__(kBlock) coarse_relayout_kernel(const T* __restrict__ in, T* __restrict__ out,
                                                                  int64_t ncb, int32_t nrhs, int dir, double alpha,
                                                                  double beta, const T* __restrict__ Z) {
+  pdl_wait();
   const int64_t total = ncb * nrhs;
   const T scale = dir == 0 ? (T)(alpha / NB) : (T)1;
   const T tb = (T)beta;
@@ -687,11 +701,11 @@ static void relayout_t(const void* in, void* out, int64_t ncb, int32_t nrhs, int
   T* o = static_cast<T*>(out);
   const T* z = static_cast<const T*>(Z);
   switch (nb) {
-    case 1: coarse_relayout_kernel<T, 1><<<g, kBlock, 0, st>>>(i, o, ncb, nrhs, dir, alpha, beta, z); break;
-    case 2: coarse_relayout_kernel<T, 2><<<g, kBlock, 0, st>>>(i, o, ncb, nrhs, dir, alpha, beta, z); break;
-    case 4: coarse_relayout_kernel<T, 4><<<g, kBlock, 0, st>>>(i, o, ncb, nrhs, dir, alpha, beta, z); break;
-    case 8: coarse_relayout_kernel<T, 8><<<g, kBlock, 0, st>>>(i, o, ncb, nrhs, dir, alpha, beta, z); break;
-    case 16: coarse_relayout_kernel<T, 16><<<g, kBlock, 0, st>>>(i, o, ncb, nrhs, dir, alpha, beta, z); break;
+    case 1: launch_pdl(coarse_relayout_kernel<T, 1>, g, kBlock, 0, st, i, o, ncb, nrhs, dir, alpha, beta, z); break;
+    case 2: launch_pdl(coarse_relayout_kernel<T, 2>, g, kBlock, 0, st, i, o, ncb, nrhs, dir, alpha, beta, z); break;
+    case 4: launch_pdl(coarse_relayout_kernel<T, 4>, g, kBlock, 0, st, i, o, ncb, nrhs, dir, alpha, beta, z); break;
+    case 8: launch_pdl(coarse_relayout_kernel<T, 8>, g, kBlock, 0, st, i, o, ncb, nrhs, dir, alpha, beta, z); break;
+    case 16: launch_pdl(coarse_relayout_kernel<T, 16>, g, kBlock, 0, st, i, o, ncb, nrhs, dir, alpha, beta, z); break;
     default: fail(AMGSYM_ERR_ARG, "coarse relayout: 2^s must be at most 16");
   }
 }
@@ -715,14 +729,18 @@ void launch_hold(int32_t naps, cudaStream_t st) {
   hold_kernel<<<1, 1, 0, st>>>(std::max<int32_t>(0, std::min<int32_t>(naps, 2000)));
 }
 
-__global__ void set_value_kernel(double* dst, double v) { *dst = v; }
+__global__ void set_value_kernel(double* dst, double v) {
+  pdl_wait();
+  *dst = v;
+}
 
 void launch_set_value(double* dst, double v, cudaStream_t st) {
   count_launch();
-  set_value_kernel<<<1, 1, 0, st>>>(dst, v);
+  launch_pdl(set_value_kernel, 1, 1, 0, st, dst, v);
 }
 
 __global__ void init_scalars_kernel(DevScalars sc, int32_t nrhs, int32_t nb) {
+  pdl_wait();
   __shared__ int n_act;
   if (threadIdx.x == 0) n_act = 0;
   __syncthreads();
@@ -748,7 +766,7 @@ __global__ void init_scalars_kernel(DevScalars sc, int32_t nrhs, int32_t nb) {
 
 void launch_init_scalars(const DevScalars& sc, int32_t nrhs, int32_t nb, cudaStream_t st) {
   count_launch();
-  init_scalars_kernel<<<1, kBlock, 0, st>>>(sc, nrhs, nb);
+  launch_pdl(init_scalars_kernel, 1, kBlock, 0, st, sc, nrhs, nb);
 }
 
 // ---------------------------------------------------------------------------

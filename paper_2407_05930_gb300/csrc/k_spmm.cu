@@ -40,6 +40,7 @@ namespace amgsym {
 template <typename MT, typename XT, typename OT, int CPT, int KL, bool HAS_DOT, bool HAS_IFACE, bool DIA>
 __global__ void __launch_bounds__(kBlock, spmm_min_blocks<XT, CPT, HAS_DOT, HAS_IFACE, DIA>()) spmm_kernel(SpmmArgs a) {
   using DT = typename AccOf<XT>::type;
+  pdl_wait();
   if (a.skip && *a.skip == 0) return;  // uniform over the grid
   constexpr int E = tile_cols<CPT, KL>();
   DT dpart[E];
@@ -247,7 +248,7 @@ static void launch_k(const SpmmArgs& a, cudaStream_t st) {
   auto run = [&](auto kern, size_t smem) {
     int g = std::min(grid, resident_grid((const void*)kern, smem));
     if (dot && (int64_t)g * a.C > a.dot.sc.partial_cap) g = (int)(a.dot.sc.partial_cap / a.C);
-    kern<<<g, kBlock, smem, st>>>(a);
+    launch_dep(a.pdl, kern, g, kBlock, smem, st, a);
   };
   if (dot) {
     const size_t smem = sizeof(double) * (size_t)dot_smem_doubles(TPC * KL, rows_pb, a.C);

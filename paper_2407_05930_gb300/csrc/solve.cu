@@ -751,6 +751,7 @@ SpmmArgs make_spmm_args(const Ctx& c, const DevCsr& M, ValType mt, VecType xt, V
   }
   if (dot) a.dot = *dot;
   a.skip = c.skip;
+  a.pdl = c.pdl;
   // the dot-fused variant has its own tile where the tuner timed one
   auto it = c.D->tiles.end();
   if (dot) it = c.D->tiles.find(TileKey{M.idx, c.C, (int)mt, (int)xt, (int)ot, 1});
@@ -1602,6 +1603,7 @@ extern "C" amgsym_status amgsym_apply_reduced(amgsym_t h, const void* X_dev, voi
   const ValType mt = f64 ? VAL_F64 : VAL_F32;
   if (!D->Ainn.vals(mt)) fail(AMGSYM_ERR_STATE, "value precision not built");
   Ctx c{D, nrhs * D->nb, vt, mt, false, (cudaStream_t)stream};
+  c.pdl = false;  // one launch: nothing of this call to overlap
   spmm(c, D->Ainn, mt, vt, vt, X_dev, Y_dev, 1.0, 0.0, nullptr, true, nullptr);
   API_END
 }
