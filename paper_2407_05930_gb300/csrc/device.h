@@ -275,6 +275,8 @@ void launch_mdot(const double* V, int64_t vstride, int32_t Cv, int32_t J, const 
 // W[row][c] += sign * sum_j V_j[row][c % Cv] H[j * C + c]
 void launch_maxpy(const double* V, int64_t vstride, int32_t Cv, int32_t J, const double* H, double sign, double* W,
                   int64_t rows, int32_t C, cudaStream_t st);
+// out[row][c] = W[row][c] / sqrt(n2[c]), 0 where n2[c] <= 0 (out may be W)
+void launch_colnormalize(const double* W, const double* n2, double* out, int64_t rows, int32_t C, cudaStream_t st);
 // out[row][c] = W[row][c] s[c] (out may be W)
 void launch_colscale(const double* W, const double* s, double* out, int64_t rows, int32_t C, cudaStream_t st);
 // AMGR coarse step layouts (k_misc.cu): dir 0 from the transformed

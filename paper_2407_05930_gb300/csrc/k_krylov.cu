@@ -134,6 +134,23 @@ __global__ void __launch_bounds__(kBlock) colscale_kernel(const double* __restri
     out[e] = W[e] * s[e % C];
 }
 
+// out[row][c] = W[row][c] * (1 / sqrt(n2[c])), 0 where n2[c] <= 0: the factors
+// once per block (C <= kBlock).
+__global__ void __launch_bounds__(kBlock) colnormalize_kernel(const double* __restrict__ W,
+                                                              const double* __restrict__ n2, double* __restrict__ out,
+                                                              int64_t rows, int32_t C) {
+  pdl_wait();
+  __shared__ double s[kBlock];
+  if ((int)threadIdx.x < C) {
+    const double n = sqrt(fmax(0.0, n2[threadIdx.x]));
+    s[threadIdx.x] = n > 0.0 ? 1.0 / n : 0.0;
+  }
+  __syncthreads();
+  const int64_t total = rows * C;
+  for (int64_t e = blockIdx.x * (int64_t)kBlock + threadIdx.x; e < total; e += (int64_t)gridDim.x * kBlock)
+    out[e] = W[e] * s[e % C];
+}
+
 int grid_elems(int64_t total) {
   return (int)std::max<int64_t>(1, std::min<int64_t>((total + kBlock - 1) / kBlock, max_grid_blocks()));
 }
@@ -159,6 +176,11 @@ void launch_maxpy(const double* V, int64_t vstride, int32_t Cv, int32_t J, const
   if (J <= 0) return;
   count_launch();
   launch_pdl(maxpy_kernel, grid_elems(rows * C), kBlock, 0, st, V, vstride, Cv, J, H, sign, W, rows, C);
+}
+
+void launch_colnormalize(const double* W, const double* n2, double* out, int64_t rows, int32_t C, cudaStream_t st) {
+  count_launch();
+  launch_pdl(colnormalize_kernel, grid_elems(rows * C), kBlock, 0, st, W, n2, out, rows, C);
 }
 
 void launch_colscale(const double* W, const double* s, double* out, int64_t rows, int32_t C, cudaStream_t st) {
