@@ -146,6 +146,17 @@ struct DotArgs {
   ConvParams cp{};
 };
 
+// Epilogue of an SpMM: Y = alpha (M X) + beta Z.  The form and the FP32 factors
+// are fixed on the host: an FP64 compare or conversion in the row loop issues
+// at the FP64 rate (2 lanes per clock per SM), for FP32 products too.
+enum SpmmEpi {
+  EPI_SUM = 0,        // alpha = 1, beta = 0
+  EPI_SCALE = 1,      // beta = 0
+  EPI_RESIDUAL = 2,   // alpha = -1, beta = 1: Z - M X
+  EPI_UPDATE = 3,     // beta = 1
+  EPI_GENERAL = 4
+};
+
 struct SpmmArgs {
   int32_t rows = 0, C = 0;
   const int32_t* ptr = nullptr;
@@ -154,7 +165,18 @@ struct SpmmArgs {
   const void* X = nullptr;
   void* Y = nullptr;
   const void* Z = nullptr;  // epilogue operand (XT)
-  double alpha = 1.0, beta = 0.0;
+  double alpha = 1.0, beta = 0.0;  // set by set_factors
+  float alpha_f = 1.f, beta_f = 0.f;
+  int32_t epi = EPI_SUM;
+  void set_factors(double al, double be) {
+    alpha = al;
+    beta = be;
+    alpha_f = (float)al;
+    beta_f = (float)be;
+    epi = be == 0.0 ? (al == 1.0 ? EPI_SUM : EPI_SCALE)
+          : be == 1.0 ? (al == -1.0 ? EPI_RESIDUAL : EPI_UPDATE)
+                      : EPI_GENERAL;
+  }
   // Interface correction (NULL mask = none).
   const uint32_t* imask = nullptr;
   const int32_t* iprefix = nullptr;

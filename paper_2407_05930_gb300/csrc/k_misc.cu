@@ -104,7 +104,10 @@ __device__ __forceinline__ double scale_down(double v) {
   const int hi = __double2hiint(v);
   const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;
   if (e - (S + 1u) < 0x7ffu - (S + 1u)) return __hiloint2double(hi - (S << 20), __double2loint(v));
-  return v * (1.0 / (double)(1 << S));
+  // volatile: the compiler would compute it beside the other and select
+  double r;
+  asm volatile("mul.rn.f64 %0, %1, %2;" : "=d"(r) : "d"(v), "d"(1.0 / (double)(1 << S)));
+  return r;
 }
 
 template <int S>
@@ -666,6 +669,7 @@ __global__ void __launch_bounds__(kBlock) coarse_relayout_kernel(const T* __rest
   const int64_t total = ncb * nrhs;
   const T scale = dir == 0 ? (T)(alpha / NB) : (T)1;
   const T tb = (T)beta;
+  const bool add = beta != 0.0;  // once: an FP64 compare per value would bound the kernel
   for (int64_t t = blockIdx.x * (int64_t)kBlock + threadIdx.x; t < total; t += (int64_t)gridDim.x * kBlock) {
     const int64_t l = t / nrhs;
     const int32_t r = (int32_t)(t - l * nrhs);
@@ -686,7 +690,7 @@ __global__ void __launch_bounds__(kBlock) coarse_relayout_kernel(const T* __rest
     for (int j = 0; j < NB; ++j) {
       if (dir == 0) {
         const int64_t o = (l * NB + j) * nrhs + r;
-        out[o] = beta != 0.0 ? scale * v[j] + tb * Z[o] : scale * v[j];
+        out[o] = add ? scale * v[j] + tb * Z[o] : scale * v[j];
       } else {
         out[l * nrhs * NB + (int64_t)r * NB + j] = v[j];
       }

@@ -710,8 +710,7 @@ SpmmArgs make_spmm_args(const Ctx& c, const DevCsr& M, ValType mt, VecType xt, V
   a.X = X;
   a.Y = Y;
   a.Z = Z;
-  a.alpha = alpha;
-  a.beta = beta;
+  a.set_factors(alpha, beta);
   if (iface && c.D->iface.mask) {
     a.imask = c.D->iface.mask;
     a.iprefix = c.D->iface.prefix;

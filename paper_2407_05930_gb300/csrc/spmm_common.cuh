@@ -271,27 +271,34 @@ __device__ __forceinline__ void row_epilogue(const SpmmArgs& a, int row, int c0,
                                              const Vec<XT, CPT>& zpre, bool use_zpre, const Vec<XT, CPT>& wpre,
                                              bool use_wpre, DT (&dpart)[CPT]) {
   const int C = a.C;
-  const CT alpha = (CT)a.alpha, beta = (CT)a.beta;
+  CT alpha, beta;
+  if constexpr (sizeof(CT) == 8) {
+    alpha = a.alpha;
+    beta = a.beta;
+  } else {
+    alpha = a.alpha_f;
+    beta = a.beta_f;
+  }
   // Y may alias Z (in-place update z += ...); each row reads Z before writing Y.
   OT* Y = static_cast<OT*>(a.Y);
   Vec<OT, CPT> out;
-  if (a.beta != 0.0) {
+  if (a.epi >= EPI_RESIDUAL) {
     // the epilogue operand as loaded early by the caller (use_zpre), else now;
     // passed by value so that it stays in registers
     const Vec<XT, CPT> zv = use_zpre ? zpre : ldx<XT, CPT, COH>(static_cast<const XT*>(a.Z) + (int64_t)row * C + c0);
-    // FP64: the factors +-1 of residuals and updates without their multiply
-    // (the same rounding: z - acc = fma(-1, acc, 1 * z))
-    if (sizeof(CT) == 8 && a.beta == 1.0 && a.alpha == -1.0) {
+    // the factors +-1 of residuals and updates take no multiply (the same
+    // rounding: z - acc = fma(-1, acc, 1 * z))
+    if (a.epi == EPI_RESIDUAL) {
 #pragma unroll
       for (int q = 0; q < CPT; ++q) acc[q] = (CT)zv.v[q] - acc[q];
-    } else if (sizeof(CT) == 8 && a.beta == 1.0) {
+    } else if (a.epi == EPI_UPDATE) {
 #pragma unroll
       for (int q = 0; q < CPT; ++q) acc[q] = fma(alpha, acc[q], (CT)zv.v[q]);
     } else {
 #pragma unroll
       for (int q = 0; q < CPT; ++q) acc[q] = fma(alpha, acc[q], beta * (CT)zv.v[q]);
     }
-  } else if (sizeof(CT) != 8 || a.alpha != 1.0) {
+  } else if (a.epi == EPI_SCALE) {
 #pragma unroll
     for (int q = 0; q < CPT; ++q) acc[q] = alpha * acc[q];
   }
@@ -503,7 +510,7 @@ __device__ __forceinline__ void spmm_tile(const SpmmArgs& a, int first_slot, int
       // interface flag word and epilogue operand loaded with the row pointers,
       // off the critical path of the gathers
       const uint32_t iface_word = (HAS_IFACE && own) ? __ldg(a.imask + (row >> 5)) : 0u;
-      if ((ZPF || DPF) && own && a.beta != 0.0) zpre = ldx<XT, E, COH>(Z + (int64_t)row * C + ec0);
+      if ((ZPF || DPF) && own && a.epi >= EPI_RESIDUAL) zpre = ldx<XT, E, COH>(Z + (int64_t)row * C + ec0);
       if (DPF && own && a.dot.mode == DOT_WY)
         wpre = ldx<XT, E, COH>(static_cast<const XT*>(a.dot.W) + (int64_t)row * C + ec0);
       if (DIA)
@@ -514,7 +521,7 @@ __device__ __forceinline__ void spmm_tile(const SpmmArgs& a, int first_slot, int
     }
     combine_lanes<CPT, KL, CT>(t, acc);
     if (own && !flagged)
-      epilogue(row, acc, zpre, (ZPF || DPF) && a.beta != 0.0, wpre, DPF && a.dot.mode == DOT_WY);
+      epilogue(row, acc, zpre, (ZPF || DPF) && a.epi >= EPI_RESIDUAL, wpre, DPF && a.dot.mode == DOT_WY);
   }
   if (HAS_IFACE) {
     // the flagged rows, with their couplings

@@ -150,7 +150,7 @@ __global__ void __launch_bounds__(kBlock, 2) stencil_kernel(SpmmArgs a) {
       const int row = base + gxy * z;
       // this plane's epilogue operands, in flight across the barrier
       V zpre, wpre;
-      const bool use_z = a.beta != 0.0, use_w = HAS_DOT && a.dot.mode == DOT_WY;
+      const bool use_z = a.epi >= EPI_RESIDUAL, use_w = HAS_DOT && a.dot.mode == DOT_WY;
       if (use_z) zpre = ldv<XT, CPT>(static_cast<const XT*>(a.Z) + (int64_t)row * CPT);
       if (use_w) wpre = ldv<XT, CPT>(static_cast<const XT*>(a.dot.W) + (int64_t)row * CPT);
       const uint32_t iface_word = HAS_IFACE ? __ldg(a.imask + (row >> 5)) : 0u;
