@@ -86,26 +86,37 @@ __device__ __forceinline__ void dot_finalize_rhs(const DotArgs& d, const double*
 // threads to terms, so the order of additions, and the result, never varies
 // from run to run.  Shared scratch (dynamic): dot_smem_doubles(...).
 //
-// What bounds it: FP64 adds issue at 2 lanes per clock per SM here (16 cycles
-// a warp instruction) and one dependent add takes longer than a shared load,
-// so the tail of a fused dot is the number of FP64 add instructions per warp
-// plus the chains of dependent adds, not the bytes.  Hence: a warp combines
-// its row slots by halving exchanges (lane pairs swap half of their columns,
-// so 8 columns over 32 lanes take 4 + 2 + 1 + 1 + 1 = 9 adds a lane, not
-// 8 x 5 = 40), and every later stage sums a few interleaved chains.
-// Measured on whole solves to 1e-12: FP64 2D 64x64 (C = 2, three dots an
-// iteration) 4.05 -> 2.96 ms, mixed 256^3 (C = 8) 107.1 -> 103.9 ms, against
-// full butterflies of every column and one thread per column summing up to 128
-// slices.
+// What bounds it: FP64 adds and conversions issue at 2 lanes per clock per SM
+// here (16 cycles a warp instruction), so the tail of a fused dot is the number
+// of FP64 instructions per SM plus the chains of dependent adds and of L2 round
+// trips, not the bytes.  Hence:
+//  * FP64 partials: a warp combines its row slots by halving exchanges (lane
+//    pairs swap half of their columns: 4 + 2 + 1 + 1 + 1 = 9 adds a lane for 8
+//    columns, not 8 x 5 = 40).
+//  * FP32 partials go to shared memory as they are; kBlock threads sum them as
+//    an unevaluated FP32 pair (error-free additions, the errors summed beside
+//    the sum: 48 bits, the partials themselves carry 24) and convert the pair
+//    once, instead of a conversion and an FP64 add for every partial.
+//  * The block partials: eight loads in flight per thread; from 16 columns on in
+//    two levels, so that the last block does not add nslots x C values alone.
+// Before, from a block's last product to the end of the kernel (456 blocks, FP32):
+// 6.2 us at 8 columns, 12.5 at 24, 10.0 at 32, of which the last block's sum of
+// the block partials 3.0, 6.3 and 7.5; a mixed solve runs three of these an
+// iteration (128^3 at 32 columns, to 1e-12: 31.8 -> 30.9 ms; 256^3: 100.5 -> 99.9).
 __host__ __device__ inline bool dot_shuffles(int S) { return S > 0 && (S & (S - 1)) == 0 && S <= 32; }
 
-// Lines of per-column partials a block leaves in shared memory: one per warp
-// when the S lanes of a row slot divide a warp, else one per row slot.
+// Lines of per-column FP64 partials a block leaves in shared memory: one per
+// warp when the S lanes of a row slot divide a warp, else one per row slot.
 __host__ __device__ inline int dot_lines(int S, int rows_pb) { return dot_shuffles(S) ? kBlock / 32 : rows_pb; }
 
-__host__ __device__ inline int dot_smem_doubles(int S, int rows_pb, int C) {
-  return dot_lines(S, rows_pb) * C + kBlock + C;
+// Shared scratch: the lines (FP64), or the FP32 partials column by column (an
+// odd pitch spreads the columns of a row slot over the banks); then the sums.
+__host__ __device__ inline int dot_pitch(int rows_pb) { return rows_pb | 1; }
+__host__ __device__ inline int dot_area(int S, int rows_pb, int C) {
+  const int f64 = dot_lines(S, rows_pb) * C, f32 = (C * dot_pitch(rows_pb) + 1) / 2;
+  return (f64 > f32 ? f64 : f32) + C;
 }
+__host__ __device__ inline int dot_smem_doubles(int S, int rows_pb, int C) { return dot_area(S, rows_pb, C) + kBlock; }
 
 // Steps K.. of the halving exchange over the lanes lane ^ (S << K): v[0 .. NV)
 // holds columns sub .. sub + NV - 1 of the thread's CPT.  `dup`: this lane's
@@ -132,10 +143,51 @@ __device__ __forceinline__ void dot_exchange(double (&v)[CPT], int off, int lane
   }
 }
 
-// The block's threads' partials as lines of C columns in sm (unsynchronised).
+// out[c] = sum over sl < n of red[sl * C + c], halving n: log2(n) dependent
+// adds.  Starts and ends with a barrier.
+__device__ __forceinline__ void dot_fold(int n, int C, double* red, double* out) {
+  const int c = threadIdx.x % C, sl = threadIdx.x / C;
+  while (n > 1) {
+    const int h = (n + 1) >> 1;
+    __syncthreads();
+    if (sl < n - h) red[sl * C + c] += red[(sl + h) * C + c];
+    n = h;
+  }
+  __syncthreads();
+  if (sl == 0) out[c] = red[c];
+  __syncthreads();
+}
+
+// out[c] = sum of `count` lines of src (stride C; GLOBAL: written by other
+// blocks, read through L2), for the whole block: thread t sums the lines
+// t / C, t / C + slices, ... of column t % C in four chains, eight loads in
+// flight; the slices are folded in red (kBlock doubles).
+template <bool GLOBAL>
+__device__ __forceinline__ void dot_sum_lines(const double* src, int count, int C, double* red, double* out) {
+  const int c = threadIdx.x % C, sl = threadIdx.x / C;
+  auto ld = [&](int r) { return GLOBAL ? __ldcg(src + (int64_t)r * C + c) : src[r * C + c]; };
+  constexpr int U = GLOBAL ? 8 : 4;
+  // few lines in shared memory: one thread per column, nothing to fold
+  const int slices = !GLOBAL && count <= 8 ? 1 : min((int)blockDim.x / C, count);
+  if (sl < slices) {
+    double t[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int r = sl; r < count; r += U * slices) {
+      double v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) v[u] = r + u * slices < count ? ld(r + u * slices) : 0.0;
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+        if (r + u * slices < count) t[u & 3] += v[u];
+    }
+    red[sl * C + c] = (t[0] + t[1]) + (t[2] + t[3]);
+  }
+  dot_fold(slices, C, red, out);
+}
+
+// The block's sum per column of FP64 partials.
 template <int CPT>
-__device__ __forceinline__ void dot_block_lines(double (&part)[CPT], int c0, bool has_cols, int rloc, int S, int C,
-                                                double* sm) {
+__device__ __forceinline__ void dot_block_sum(double (&part)[CPT], int c0, bool has_cols, int rloc, int rows_pb, int S,
+                                              int C, double* sm, double* red, double* out) {
   if (dot_shuffles(S)) {
     const int lane = threadIdx.x & 31;
     int sub = 0;
@@ -153,46 +205,45 @@ __device__ __forceinline__ void dot_block_lines(double (&part)[CPT], int c0, boo
 #pragma unroll
     for (int q = 0; q < CPT; ++q) sm[rloc * C + c0 + q] = part[q];
   }
+  __syncthreads();
+  dot_sum_lines<false>(sm, dot_lines(S, rows_pb), C, red, out);
 }
 
-// out[c] = sum of `count` lines of src (stride C; GLOBAL: written by other
-// blocks, read through L2), for the whole block: thread t sums the lines
-// t / C, t / C + slices, ... of column t % C in four chains, then the slices
-// are added in shared memory (red: kBlock doubles) by four chains again.
-// Synchronises before out may be read.
-template <bool GLOBAL>
-__device__ __forceinline__ void dot_sum_lines(const double* src, int count, int C, double* red, double* out) {
-  const int c = threadIdx.x % C, sl = threadIdx.x / C;
-  auto ld = [&](int r) { return GLOBAL ? __ldcg(src + (int64_t)r * C + c) : src[r * C + c]; };
-  // few lines: one thread per column, no second stage
-  const int slices = count <= 8 ? 1 : min((int)blockDim.x / C, count);
-  if (sl < slices) {
-    double t[4] = {0.0, 0.0, 0.0, 0.0};
-    int r = sl;
-    for (; r + 3 * slices < count; r += 4 * slices) {
+// The same of FP32 partials, as FP32 pairs: hi + x with its exact error (Knuth's
+// two-sum) added to lo.  Partials of 2^90 or more, infinities and NaN are
+// summed in FP64 (the pair could overflow, or turn an infinity into a NaN).
+template <int CPT>
+__device__ __forceinline__ void dot_block_sum(float (&part)[CPT], int c0, bool has_cols, int rloc, int rows_pb, int S,
+                                              int C, double* sm, double* red, double* out) {
+  float* f = reinterpret_cast<float*>(sm);
+  const int pitch = dot_pitch(rows_pb);
+  if (has_cols) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u) t[u] += ld(r + u * slices);
-    }
-#pragma unroll
-    for (int u = 0; u < 3; ++u)
-      if (r + u * slices < count) t[u] += ld(r + u * slices);
-    const double v = (t[0] + t[1]) + (t[2] + t[3]);
-    if (slices == 1)
-      out[c] = v;
-    else
-      red[sl * C + c] = v;
-  }
-  // halve the slices until one is left: log2(slices) dependent adds
-  for (int n = slices; n > 1;) {
-    const int h = (n + 1) >> 1;
-    __syncthreads();
-    if (sl < n - h) red[sl * C + c] += red[(sl + h) * C + c];
-    n = h;
-  }
-  if (slices > 1) {
-    if (sl == 0) out[c] = red[c];
+    for (int q = 0; q < CPT; ++q) f[(c0 + q) * pitch + rloc] = part[q];
   }
   __syncthreads();
+  const int nsl = min(kBlock / C, rows_pb);
+  const int c = threadIdx.x / nsl, sl = threadIdx.x - c * nsl;
+  if (c < C) {
+    const float* col = f + c * pitch;
+    float hi = 0.f, lo = 0.f;
+    bool big = false;
+    for (int r = sl; r < rows_pb; r += nsl) {
+      const float x = col[r];
+      big |= !(fabsf(x) < 0x1p90f);
+      const float t = __fadd_rn(hi, x);
+      const float xr = __fsub_rn(t, hi);
+      lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, xr)), __fsub_rn(x, xr)));
+      hi = t;
+    }
+    double v = (double)hi + (double)lo;
+    if (big) {
+      v = 0.0;
+      for (int r = sl; r < rows_pb; r += nsl) v += (double)col[r];
+    }
+    red[sl * C + c] = v;
+  }
+  dot_fold(nsl, C, red, out);
 }
 
 // The CG scalars of every column, then of every right-hand side.
@@ -212,66 +263,69 @@ __device__ __forceinline__ void dot_finalize(const DotArgs& d, const double* col
   }
 }
 
-template <int CPT>
-__device__ __forceinline__ void block_dot(const DotArgs& d, double (&part)[CPT], int c0, bool has_cols,
-                                          int rloc, int rows_pb, int S, int C, double* sm, int slot, int nslots,
-                                          double* partials, unsigned* ticket) {
-  const int lines = dot_lines(S, rows_pb);
-  double* red = sm + lines * C;
-  dot_block_lines<CPT>(part, c0, has_cols, rloc, S, C, sm);
-  __syncthreads();
-  dot_sum_lines<false>(sm, lines, C, red, partials + (int64_t)slot * C);
-  __shared__ unsigned is_last;
+// One of n arrivals at a ticket: whether this block is the last.  The block's
+// stores, made visible to thread 0 by the barrier before, are released with its
+// arrival (cumulativity) and acquired by the last block.
+__device__ __forceinline__ bool dot_arrive(unsigned* ticket, int n) {
+  __shared__ unsigned last;
   if (threadIdx.x == 0) {
-    // the block's stores, made visible to this thread by the barrier, are
-    // released with its arrival (cumulativity), and acquired by the last block
     __threadfence();
-    is_last = (atomicAdd(ticket, 1u) == (unsigned)nslots - 1u) ? 1u : 0u;
+    last = (atomicAdd(ticket, 1u) == (unsigned)n - 1u) ? 1u : 0u;
     __threadfence();
   }
   __syncthreads();
-  if (!is_last) return;
-  double* colsum = sm;  // [C] (the line area is free now)
-  dot_sum_lines<true>(partials, nslots, C, red, colsum);
-  dot_finalize(d, colsum, C);
-  if (threadIdx.x == 0) *ticket = 0u;
-  __syncthreads();  // the block may go on to reuse the shared scratch
+  const bool l = last != 0u;
+  __syncthreads();  // before another arrival writes it
+  return l;
 }
 
-// Two-level variant for the batched kernels (see BDot): any number of items
-// per problem, each reduction stage reading at most 32 lines per column.
-template <int CPT>
-__device__ __forceinline__ void block_dot2(const DotArgs& d, double (&part)[CPT], int c0, bool has_cols, int rloc,
+// Two levels: blocks (slots) leave partials[slot]; the last of each chunk of 32
+// slots sums them into chunk_partials[chunk]; the last chunk sums those and
+// finalises.  Any number of slots, each stage reading at most 32 lines a column
+// (up to 1024 slots).
+template <int CPT, typename DT>
+__device__ __forceinline__ void block_dot2(const DotArgs& d, DT (&part)[CPT], int c0, bool has_cols, int rloc,
                                            int rows_pb, int S, int C, double* sm, int slot, const BDot& bd) {
-  const int lines = dot_lines(S, rows_pb);
-  double* red = sm + lines * C;
-  dot_block_lines<CPT>(part, c0, has_cols, rloc, S, C, sm);
-  __syncthreads();
-  dot_sum_lines<false>(sm, lines, C, red, bd.partials + (int64_t)slot * C);
-  __shared__ unsigned last_chunk, last_all;
+  double* red = sm + dot_area(S, rows_pb, C);
+  dot_block_sum<CPT>(part, c0, has_cols, rloc, rows_pb, S, C, sm, red, bd.partials + (int64_t)slot * C);
   const int chunk = slot >> 5;
   const int nch = (bd.nslots + 31) >> 5;
   const int in_chunk = min(32, bd.nslots - chunk * 32);
-  if (threadIdx.x == 0) {
-    __threadfence();
-    last_chunk = (atomicAdd(bd.chunk_tickets + chunk, 1u) == (unsigned)in_chunk - 1u) ? 1u : 0u;
-    __threadfence();
-  }
-  __syncthreads();
-  if (!last_chunk) return;
+  if (!dot_arrive(bd.chunk_tickets + chunk, in_chunk)) return;
   dot_sum_lines<true>(bd.partials + (int64_t)chunk * 32 * C, in_chunk, C, red, bd.chunk_partials + (int64_t)chunk * C);
-  if (threadIdx.x == 0) {
-    bd.chunk_tickets[chunk] = 0u;
-    __threadfence();
-    last_all = (atomicAdd(bd.ticket, 1u) == (unsigned)nch - 1u) ? 1u : 0u;
-    __threadfence();
-  }
-  __syncthreads();
-  if (!last_all) return;
-  double* colsum = sm;
+  if (threadIdx.x == 0) bd.chunk_tickets[chunk] = 0u;
+  if (!dot_arrive(bd.ticket, nch)) return;
+  double* colsum = sm;  // [C] (the partials' area is free now)
   dot_sum_lines<true>(bd.chunk_partials, nch, C, red, colsum);
   dot_finalize(d, colsum, C);
   if (threadIdx.x == 0) *bd.ticket = 0u;
+  __syncthreads();  // the block may go on to reuse the shared scratch
+}
+
+// The grid's dot of one problem (slot = block): one level below 16 columns,
+// where the last block's nslots x C adds are shorter than a second arrival.
+template <int CPT, typename DT>
+__device__ __forceinline__ void block_dot(const DotArgs& d, DT (&part)[CPT], int c0, bool has_cols, int rloc,
+                                          int rows_pb, int S, int C, double* sm) {
+  const DevScalars& sc = d.sc;
+  const int slot = blockIdx.x, nslots = gridDim.x;
+  if (C >= 16 && nslots > 32) {
+    BDot bd;
+    bd.partials = sc.partials;
+    bd.chunk_partials = sc.partials + sc.partial_cap;
+    bd.ticket = sc.ticket;
+    bd.chunk_tickets = sc.ticket + 1;
+    bd.nslots = nslots;
+    block_dot2<CPT, DT>(d, part, c0, has_cols, rloc, rows_pb, S, C, sm, slot, bd);
+    return;
+  }
+  double* red = sm + dot_area(S, rows_pb, C);
+  dot_block_sum<CPT>(part, c0, has_cols, rloc, rows_pb, S, C, sm, red, sc.partials + (int64_t)slot * C);
+  if (!dot_arrive(sc.ticket, nslots)) return;
+  double* colsum = sm;  // [C] (the partials' area is free now)
+  dot_sum_lines<true>(sc.partials, nslots, C, red, colsum);
+  dot_finalize(d, colsum, C);
+  if (threadIdx.x == 0) *sc.ticket = 0u;
   __syncthreads();
 }
 

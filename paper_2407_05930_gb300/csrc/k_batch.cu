@@ -39,11 +39,8 @@ __global__ void __launch_bounds__(kBlock, (DIA && HAS_DOT) || sizeof(XT) == 8 ? 
     spmm_tile<MT, XT, OT, CPT, KL, HAS_DOT, HAS_IFACE, DIA>(a, bi.first_slot, 1, bi.row_end, dpart, false);
     if (HAS_DOT) {
       const TileLayout t = tile_layout<CPT, KL>(a.C);
-      double part[E];
-#pragma unroll
-      for (int q = 0; q < E; ++q) part[q] = t.own ? (double)dpart[q] : 0.0;
       const BDot bd = dots[bi.arg];
-      block_dot2<E>(a.dot, part, t.ec0, t.own, t.g, t.rows_pb, t.S, a.C, sm, bi.slot, bd);
+      block_dot2<E, DT>(a.dot, dpart, t.ec0, t.own, t.g, t.rows_pb, t.S, a.C, sm, bi.slot, bd);
     }
   }
 }
@@ -216,11 +213,8 @@ __global__ void __launch_bounds__(kBlock) vec_batch_kernel(const UpdArgs* __rest
       }
     }
     if (OP == BOP_UPDATE1) {
-      double pd[CPT];
-#pragma unroll
-      for (int k = 0; k < CPT; ++k) pd[k] = has_cols ? (double)part[k] : 0.0;
       const BDot bd = dots[bi.arg];
-      block_dot2<CPT>(a.dot, pd, c0, has_cols, rloc, rows_pb, TPR, C, sm, bi.slot, bd);
+      block_dot2<CPT, DT>(a.dot, part, c0, has_cols, rloc, rows_pb, TPR, C, sm, bi.slot, bd);
     }
   }
 }

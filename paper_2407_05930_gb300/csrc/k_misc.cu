@@ -311,11 +311,7 @@ __global__ void __launch_bounds__(kBlock) cg_update1_kernel(int64_t rows, int32_
   }
   if (HAS_DOT) {
     extern __shared__ double sm[];
-    double pd[CPT];
-#pragma unroll
-    for (int k = 0; k < CPT; ++k) pd[k] = has_cols ? (double)part[k] : 0.0;
-    block_dot<CPT>(dot, pd, c0, has_cols, rloc, rows_pb, TPR, C, sm, blockIdx.x, gridDim.x, dot.sc.partials,
-                   dot.sc.ticket);
+    block_dot<CPT, DT>(dot, part, c0, has_cols, rloc, rows_pb, TPR, C, sm);
   }
 }
 
@@ -526,12 +522,8 @@ __global__ void __launch_bounds__(kBlock) dot_kernel(int64_t rows, int32_t C, co
 #pragma unroll
       for (int k = 0; k < CPT; ++k) acc[k] = fma((DT)av.v[k], (DT)bv.v[k], acc[k]);
     }
-  double part[CPT];
-#pragma unroll
-  for (int k = 0; k < CPT; ++k) part[k] = has_cols ? (double)acc[k] : 0.0;
   extern __shared__ double sm[];
-  block_dot<CPT>(dot, part, c0, has_cols, rloc, rows_pb, TPR, C, sm, blockIdx.x, gridDim.x, dot.sc.partials,
-                 dot.sc.ticket);
+  block_dot<CPT, DT>(dot, acc, c0, has_cols, rloc, rows_pb, TPR, C, sm);
 }
 
 template <typename T, int CPT>

@@ -53,11 +53,7 @@ __global__ void __launch_bounds__(kBlock, spmm_min_blocks<XT, CPT, HAS_DOT, HAS_
   if (HAS_DOT) {
     const TileLayout t = tile_layout<CPT, KL>(a.C);
     extern __shared__ double sm[];
-    double part[E];
-#pragma unroll
-    for (int q = 0; q < E; ++q) part[q] = t.own ? (double)dpart[q] : 0.0;
-    block_dot<E>(a.dot, part, t.ec0, t.own, t.g, t.rows_pb, t.S, a.C, sm, blockIdx.x, gridDim.x, a.dot.sc.partials,
-                 a.dot.sc.ticket);
+    block_dot<E, DT>(a.dot, dpart, t.ec0, t.own, t.g, t.rows_pb, t.S, a.C, sm);
   }
 }
 

@@ -599,9 +599,12 @@ void alloc_scalars(Device* D, DevScalars& sc, int32_t C, int32_t nrhs) {
   sc.active = dalloc<int32_t>(D->work_owned, C);
   sc.status = dalloc<int32_t>(D->work_owned, 4);
   sc.partial_cap = (int64_t)max_grid_blocks() * C;
-  sc.partials = dalloc<double>(D->work_owned, sc.partial_cap);
-  sc.ticket = dalloc<unsigned>(D->work_owned, 1);
-  CK(cudaMemset(sc.ticket, 0, sizeof(unsigned)));
+  // the block partials, then the sums of chunks of 32 blocks; the ticket, then
+  // the chunks' (block_dot)
+  const int64_t chunks = (max_grid_blocks() + 31) / 32;
+  sc.partials = dalloc<double>(D->work_owned, sc.partial_cap + chunks * C);
+  sc.ticket = dalloc<unsigned>(D->work_owned, 1 + chunks);
+  CK(cudaMemset(sc.ticket, 0, sizeof(unsigned) * (size_t)(1 + chunks)));
   CK(cudaMemset(sc.status, 0, 4 * sizeof(int32_t)));
 }
 

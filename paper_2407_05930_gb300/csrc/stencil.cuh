@@ -192,11 +192,7 @@ __global__ void __launch_bounds__(kBlock, 2) stencil_kernel(SpmmArgs a) {
     }
   }
   if (HAS_DOT) {
-    double part[CPT];
-#pragma unroll
-    for (int q = 0; q < CPT; ++q) part[q] = (double)dpart[q];
-    block_dot<CPT>(a.dot, part, 0, true, threadIdx.x, kBlock, 1, a.C, dsm, blockIdx.x, gridDim.x, a.dot.sc.partials,
-                   a.dot.sc.ticket);
+    block_dot<CPT, DT>(a.dot, dpart, 0, true, threadIdx.x, kBlock, 1, a.C, dsm);
   }
 }
 
