@@ -221,7 +221,7 @@ struct SpmmArgs {
   const uint16_t* lidx = nullptr;
   // Sliced form of a CSR matrix (nslices > 0; see DevCsr): used by
   // launch_spmm for products without a dot or interface at one vector of C
-  // columns per thread with at most 4 entry lanes, else the CSR kernel runs.
+  // columns per thread, else the CSR kernel runs.
   int32_t nslices = 0;
   const int32_t* sptr = nullptr;
   const int32_t* srow = nullptr;

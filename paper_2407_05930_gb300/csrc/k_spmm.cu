@@ -297,13 +297,14 @@ static void launch_t(const SpmmArgs& a, cudaStream_t st) {
     }
     return;
   }
-  if (a.nslices > 0 && a.dot.mode == DOT_NONE && !a.imask && kl <= 4 && sell_lanes_ok<XT>(a.C)) {
-    if (kl == 1)
-      launch_s<MT, XT, OT, 1>(a, st);
-    else if (kl == 2)
-      launch_s<MT, XT, OT, 2>(a, st);
-    else
-      launch_s<MT, XT, OT, 4>(a, st);
+  if (a.nslices > 0 && a.dot.mode == DOT_NONE && !a.imask && sell_lanes_ok<XT>(a.C)) {
+    switch (kl) {
+      case 1: launch_s<MT, XT, OT, 1>(a, st); break;
+      case 2: launch_s<MT, XT, OT, 2>(a, st); break;
+      case 4: launch_s<MT, XT, OT, 4>(a, st); break;
+      case 8: launch_s<MT, XT, OT, 8>(a, st); break;
+      default: launch_s<MT, XT, OT, 16>(a, st); break;
+    }
     return;
   }
   switch (kl) {
@@ -347,9 +348,8 @@ void stencil_geometry(int32_t rows, int32_t ndiag, const int32_t* off, SpmmArgs&
 
 bool spmm_uses_sell(VecType xt, VecType ot, const SpmmArgs& a) {
   if (a.nslices <= 0 || a.ndiag > 0 || a.dot.mode != DOT_NONE || a.imask || spmm_uses_halo(xt, a)) return false;
-  int cpt = 0, kl = 0;
-  spmm_resolved_tile(xt, ot, a, &cpt, &kl);
-  return kl <= 4 && (xt == VEC_F64 ? sell_lanes_ok<double>(a.C) : sell_lanes_ok<float>(a.C));
+  (void)ot;
+  return xt == VEC_F64 ? sell_lanes_ok<double>(a.C) : sell_lanes_ok<float>(a.C);
 }
 
 bool spmm_uses_stencil(ValType mt, VecType xt, VecType ot, const SpmmArgs& a) {

@@ -35,14 +35,14 @@ namespace amgsym {
 // scheduler balances slices of different widths).  The next batch's columns
 // and values load while the current batch's gathers are in flight.
 template <typename MT, typename XT, typename OT, int KL>
-__global__ void __launch_bounds__(kBlock, sizeof(XT) == 8 ? 3 : 4) sell_kernel(SpmmArgs a) {
-  static_assert(KL == 1 || KL == 2 || KL == 4, "1, 2 or 4 entry lanes");
+__global__ void __launch_bounds__(kBlock, KL > 4 ? 1 : sizeof(XT) == 8 ? 3 : 4) sell_kernel(SpmmArgs a) {
+  static_assert((KL & (KL - 1)) == 0 && KL <= 16, "1 to 16 entry lanes");
   constexpr int CPT = 16 / (int)sizeof(XT);
   using CT = typename ComputeOf<MT, XT>::type;
   using DT = typename AccOf<XT>::type;
   using V = Vec<XT, CPT>;
   if (a.skip && *a.skip == 0) return;  // uniform over the grid
-  constexpr int B = 4;                 // entries per lane per round trip (a multiple of KL)
+  constexpr int B = KL > 4 ? KL : 4;   // entries per lane per round trip (a multiple of KL)
   static_assert(B % KL == 0, "batch must keep entry i in partial i mod KL");
   const int C = a.C, TPC = C / CPT, rpw = 32 / TPC;
   const int lane = threadIdx.x & 31;
@@ -99,16 +99,15 @@ __global__ void __launch_bounds__(kBlock, sizeof(XT) == 8 ? 3 : 4) sell_kernel(S
         for (int q = 0; q < CPT; ++q) acc[u % KL][q] = fma(m[u], (CT)x[u].v[q], acc[u % KL][q]);
       }
   }
+#pragma unroll
+  for (int off = KL / 2; off >= 1; off >>= 1)
+#pragma unroll
+    for (int k = 0; k < off; ++k)
+#pragma unroll
+      for (int q = 0; q < CPT; ++q) acc[k][q] = acc[k][q] + acc[k + off][q];
   CT out[CPT];
 #pragma unroll
-  for (int q = 0; q < CPT; ++q) {
-    if (KL == 1)
-      out[q] = acc[0][q];
-    else if (KL == 2)
-      out[q] = acc[0][q] + acc[KL - 1][q];
-    else
-      out[q] = (acc[0][q] + acc[KL / 2][q]) + (acc[1 % KL][q] + acc[(KL / 2 + 1) % KL][q]);
-  }
+  for (int q = 0; q < CPT; ++q) out[q] = acc[0][q];
   DT none[CPT];  // the epilogue's dot partial: no dot here
   if (row >= 0) row_epilogue<XT, OT, CT, DT, CPT, false, false>(a, row, c0, out, V{}, false, V{}, false, none);
 }

@@ -669,37 +669,44 @@ void ensure_work(Device* D, int32_t nrhs, VecType vt) {
 // ---------------------------------------------------------------------------
 // Kernel sequencing.
 
-// Fixed tile from the row length (what the autotuner picks on the 256^3
-// workload, measured on GB300): short rows take one thread per row holding
-// two 16-byte vectors of columns (coalesced index/value loads for a warp of
-// consecutive rows); medium rows split their entries over 4 lanes; the long
-// rows of the coarse Galerkin operators over 4-16 lanes with one vector each.
+// Fixed tile from the row length and count (the timings of every candidate on
+// hierarchies of 64^3 to 256^3 grids at 8 to 32 columns, GB300).
+//
+// Columns per thread: two 16-byte vectors in FP32 (a gathered row of 8 columns
+// is one 32-byte sector), and for the diagonal-offset form; one in FP64 CSR
+// products, which are bound by FP64 issue and keep more warps that way (R at
+// 192^3 60 us against 68, A_1 138 against 147).
+// Entry lanes: rows of up to 4 entries (prolongations) are fastest with one
+// lane (P_0 at 256^3 30 us, 43 with two); up to 10, two (R_0 29.7 us, 31.4 with
+// one); up to 26, four (A_1 60.7 us, 66.3 and 68.5 with two and eight); longer
+// ones eight (A_2 23.2 us, 26.6 with four).  In FP64 one lane up to 10 entries,
+// else two: a lane's masked entries cost as much as real ones.
+// Then, while the matrix does not fill the GPU, twice the lanes: such a product
+// is a chain of dependent loads, one round per (lanes x entries in flight) of a
+// row (4505 rows of 27 entries: 3.5 us with 16 lanes, 5 with four; 676 rows:
+// 2.9 against 6 us).  The smallest split the columns too.
+constexpr int64_t kFillThreads = 240000;  // threads a doubling may reach: about one and a half resident waves
+
 Tile fixed_tile(const DevCsr& M, int32_t C, VecType xt) {
   const int V = xt == VEC_F64 ? 2 : 4;
-  const bool two = C % (2 * V) == 0 && C / (2 * V) >= 1;
-  Tile t;
+  const bool f64 = xt == VEC_F64;
   const double r = M.avg_row;
-  if (M.ndiag > 0) {  // diagonal-offset form: one lane per row, two vectors
-    t.cpt = two ? 2 * V : V;
-    t.kl = 1;
-  } else if (r < 10.0) {
-    t.cpt = two ? 2 * V : V;
-    t.kl = 1;
-  } else if (r < 32.0) {
-    t.cpt = two ? 2 * V : V;
-    t.kl = 4;
-  } else if (r < 60.0) {
-    t.cpt = V;
-    t.kl = 4;
-  } else {
-    t.cpt = V;
-    t.kl = 16;
-  }
-  if (C % t.cpt) t.cpt = (C % V == 0) ? V : (C % 2 == 0) ? 2 : 1;
+  Tile t;
+  t.cpt = C % (2 * V) == 0 && (!f64 || M.ndiag > 0) ? 2 * V : C % V == 0 ? V : C % 2 == 0 ? 2 : 1;
+  t.kl = 1;
+  // one lane per row: the diagonal-offset form, and stencil matrices kept in
+  // CSR (their sums are those of that form, bit for bit)
+  if (M.ndiag > 0 || (r < 10.0 && M.rows == M.cols)) return t;
+  if (f64)
+    t.kl = r < 10.0 ? 1 : 2;
+  else
+    t.kl = r < 4.0 ? 1 : r < 10.0 ? 2 : r < 26.0 ? 4 : 8;
   t.kl = clamp_lanes(C / t.cpt, t.kl);
+  auto threads = [&] { return (int64_t)M.rows * (C / t.cpt) * t.kl; };
+  while (r >= 4.0 && t.kl < 16 && 2 * t.kl <= r && C / t.cpt * 2 * t.kl <= 32 && 2 * threads() <= kFillThreads) t.kl *= 2;
+  if (r >= 4.0 && t.kl == 16 && t.cpt == 2 * V && C / V * 16 <= 32 && 4 * threads() <= kFillThreads) t.cpt = V;
   return t;
 }
-
 
 SpmmArgs make_spmm_args(const Ctx& c, const DevCsr& M, ValType mt, VecType xt, VecType ot, const void* X,
                         void* Y, double alpha, double beta, const void* Z, bool iface, const DotArgs* dot) {
