@@ -17,6 +17,25 @@
 
 namespace amgsym {
 
+// Makes args[arg] the block's record: copied by all threads, a word each, and
+// only when the item belongs to another problem than the last one (one thread's
+// 16-byte copies were some 30 dependent round trips an item, as long as the
+// item's own rows).  Returns whether the problem has nothing left to do.
+// 8 problems of 16 right-hand sides, to 1e-12: 317 -> 276 ms.
+template <typename A>
+__device__ __forceinline__ bool load_record(A& rec, const A* __restrict__ args, int arg, int& cur, bool& idle) {
+  if (arg != cur) {  // block-uniform
+    static_assert(sizeof(A) % 4 == 0, "record in 4-byte words");
+    __syncthreads();  // the previous item is done with the record
+    for (int w = threadIdx.x; w < (int)(sizeof(A) / 4); w += kBlock)
+      reinterpret_cast<unsigned*>(&rec)[w] = __ldg(reinterpret_cast<const unsigned*>(args + arg) + w);
+    __syncthreads();
+    cur = arg;
+    idle = rec.skip && *rec.skip == 0;
+  }
+  return idle;
+}
+
 template <typename MT, typename XT, typename OT, int CPT, int KL, bool HAS_DOT, bool HAS_IFACE, bool DIA>
 __global__ void __launch_bounds__(kBlock, (DIA && HAS_DOT) || sizeof(XT) == 8 ? 3 : 4)
     spmm_batch_kernel(const SpmmArgs* __restrict__ args, const BItem* __restrict__ items, int32_t n_items,
@@ -26,12 +45,11 @@ __global__ void __launch_bounds__(kBlock, (DIA && HAS_DOT) || sizeof(XT) == 8 ? 
   __shared__ __align__(16) unsigned char sa_raw[sizeof(SpmmArgs)];
   SpmmArgs& a = *reinterpret_cast<SpmmArgs*>(sa_raw);
   extern __shared__ double sm[];
+  int cur = -1;
+  bool idle = false;
   for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
     const BItem bi = items[it];
-    __syncthreads();  // the previous item is done with the record
-    if (threadIdx.x == 0) a = args[bi.arg];
-    __syncthreads();
-    if (a.skip && *a.skip == 0) continue;  // block-uniform
+    if (load_record(a, args, bi.arg, cur, idle)) continue;  // block-uniform
     constexpr int E = tile_cols<CPT, KL>();
     DT dpart[E];
 #pragma unroll
@@ -130,12 +148,11 @@ __global__ void __launch_bounds__(kBlock) vec_batch_kernel(const UpdArgs* __rest
   __shared__ __align__(16) unsigned char ua_raw[sizeof(UpdArgs)];
   UpdArgs& a = *reinterpret_cast<UpdArgs*>(ua_raw);
   extern __shared__ double sm[];
+  int cur = -1;
+  bool idle = false;
   for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
     const BItem bi = items[it];
-    __syncthreads();
-    if (threadIdx.x == 0) a = args[bi.arg];
-    __syncthreads();
-    if (a.skip && *a.skip == 0) continue;
+    if (load_record(a, args, bi.arg, cur, idle)) continue;
     const int C = a.C;
     const int TPR = C / CPT;
     const int rows_pb = kBlock / TPR;
