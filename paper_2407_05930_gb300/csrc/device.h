@@ -186,6 +186,7 @@ struct SpmmArgs {
   const int32_t* icol = nullptr;
   const void* ival = nullptr;  // same precision class as the accumulation
   int32_t nb = 1;
+  int32_t fblocks = 0;  // blocks of the launch that take the flagged rows (set by launch_spmm)
   // Early exit: when non-NULL and *skip == 0 (no active RHS) the kernel does
   // nothing (lets the host run one iteration ahead of its convergence check).
   const int32_t* skip = nullptr;

@@ -49,7 +49,18 @@ __global__ void __launch_bounds__(kBlock, spmm_min_blocks<XT, CPT, HAS_DOT, HAS_
   // Grid-stride over row slots: a wave of blocks sweeps one contiguous window
   // of rows, so the far neighbours one block gathers were recently brought
   // into L2 by another.
-  spmm_tile<MT, XT, OT, CPT, KL, HAS_DOT, HAS_IFACE, DIA>(a, blockIdx.x, gridDim.x, a.rows, dpart);
+  int slot = blockIdx.x, step = gridDim.x, end = a.rows, f_slot = 0, f_step = 0;
+  if (HAS_IFACE) {  // the first fblocks blocks take the flagged rows only, the others none
+    if ((int)blockIdx.x < a.fblocks) {
+      end = 0;
+      f_slot = blockIdx.x;
+      f_step = a.fblocks;
+    } else {
+      slot -= a.fblocks;
+      step -= a.fblocks;
+    }
+  }
+  spmm_tile<MT, XT, OT, CPT, KL, HAS_DOT, HAS_IFACE, DIA>(a, slot, step, end, dpart, true, f_slot, f_step);
   if (HAS_DOT) {
     const TileLayout t = tile_layout<CPT, KL>(a.C);
     extern __shared__ double sm[];
@@ -230,6 +241,23 @@ static void launch_h(const SpmmArgs& a, cudaStream_t st) {
   kern<<<g, kBlock, smem, st>>>(a);
 }
 
+// Blocks that take the flagged (interface) rows while the others run the main
+// pass.  A flagged row waits on a chain of dependent loads (row, pointer,
+// column, operand): as a second pass of every block it was a tail of 6 us after
+// the 32 us of the reduced product at 256^3 (FP32), 23 after 99 us in FP64 at
+// 192^3.  One block a slot when everything is resident at once, else their
+// share of the resident blocks, a flagged slot counted as four of the others
+// 
+static int iface_blocks(int64_t slots, int64_t fslots, int* grid, int resident) {
+  if (fslots <= 0) return 0;
+  if (slots + fslots <= resident) {
+    *grid = (int)(slots + fslots);
+    return (int)fslots;
+  }
+  const int64_t share = (int64_t)*grid * 4 * fslots / (slots + 4 * fslots);
+  return (int)std::max<int64_t>(1, std::min<int64_t>(share, *grid / 2));
+}
+
 template <typename MT, typename XT, typename OT, int CPT, int KL, bool DIA = false>
 static void launch_k(const SpmmArgs& a, cudaStream_t st) {
   const int TPC = a.C / CPT;
@@ -242,9 +270,17 @@ static void launch_k(const SpmmArgs& a, cudaStream_t st) {
   count_launch();
   // one full wave of resident blocks (the register count differs per variant)
   auto run = [&](auto kern, size_t smem) {
-    int g = std::min(grid, resident_grid((const void*)kern, smem));
+    const int res = resident_grid((const void*)kern, smem);
+    int g = std::min(grid, res);
+    SpmmArgs b = a;
+    if (ifc) {
+      const int64_t nf = ((int64_t)a.nflag + rows_pb - 1) / rows_pb;
+      if (need + nf > res) g = std::max(2, res);
+      if (dot && (int64_t)g * a.C > a.dot.sc.partial_cap) g = (int)(a.dot.sc.partial_cap / a.C);
+      b.fblocks = iface_blocks(need, nf, &g, res);
+    }
     if (dot && (int64_t)g * a.C > a.dot.sc.partial_cap) g = (int)(a.dot.sc.partial_cap / a.C);
-    launch_dep(a.pdl, kern, g, kBlock, smem, st, a);
+    launch_dep(a.pdl, kern, g, kBlock, smem, st, b);
   };
   if (dot) {
     const size_t smem = sizeof(double) * (size_t)dot_smem_doubles(TPC * KL, rows_pb, a.C);

@@ -442,14 +442,16 @@ __device__ __forceinline__ void combine_lanes(const TileLayout& t, CT (&acc)[CPT
 // flag -> prefix -> pointer -> coupling chain; then the flagged rows (about
 // 2 % of them at 256^3) are recomputed with their couplings, from the
 // compact list of flagged rows.  whole: the block's share of the whole
-// matrix (the flagged rows slotted like the rows); otherwise the block owns
-// rows [first_slot * rows_pb, row_end) alone and takes their flagged rows.
+// matrix, and of its flagged rows the slots f_slot, f_slot + f_step, ... (none
+// with f_step = 0); otherwise the block owns rows [first_slot * rows_pb,
+// row_end) alone and takes their flagged rows.
 // A flagged row's sum is the same in both designs: its entries, then its
 // couplings (entry lane 0), then the lane combination.
 template <typename MT, typename XT, typename OT, int CPT, int KL, bool HAS_DOT, bool HAS_IFACE, bool DIA = false,
           bool COH = false>
 __device__ __forceinline__ void spmm_tile(const SpmmArgs& a, int first_slot, int slot_step, int row_end,
-                                          typename AccOf<XT>::type (&dpart)[tile_cols<CPT, KL>()], bool whole = true) {
+                                          typename AccOf<XT>::type (&dpart)[tile_cols<CPT, KL>()], bool whole = true,
+                                          int f_slot = 0, int f_step = 0) {
   static_assert(!DIA || KL == 1, "the diagonal-offset form runs one entry lane per row");
   using CT = typename ComputeOf<MT, XT>::type;
   using DT = typename AccOf<XT>::type;  // per-thread dot partial type
@@ -523,11 +525,11 @@ __device__ __forceinline__ void spmm_tile(const SpmmArgs& a, int first_slot, int
     if (own && !flagged)
       epilogue(row, acc, zpre, (ZPF || DPF) && a.epi >= EPI_RESIDUAL, wpre, DPF && a.dot.mode == DOT_WY);
   }
-  if (HAS_IFACE) {
+  if (HAS_IFACE && (!whole || f_step > 0)) {
     // the flagged rows, with their couplings
     const int f_begin = whole ? 0 : flag_index(a, first_slot * rows_pb);
     const int f_end = whole ? a.nflag : flag_index(a, row_end);
-    const int fs0 = whole ? first_slot : 0, fstep = whole ? slot_step : 1;
+    const int fs0 = whole ? f_slot : 0, fstep = whole ? f_step : 1;
     for (int fb = f_begin + fs0 * rows_pb; fb < f_end; fb += fstep * rows_pb) {
       const int f = fb + g;
       const bool live = slot_ok && f < f_end;
