@@ -123,12 +123,17 @@ static void free_plans(Batch* B) {
 // Rows per item (in row slots of rows_pb rows): sized so that one wave of
 // resident blocks touches about 48 MB of the gathered vector (row_bytes per
 // row).  The far-neighbour rows a block gathers are then still in L2 from the
-// blocks working just behind it, even when the vector is larger than L2.
-static int slots_per_item(int64_t rows, int rows_pb, int64_t row_bytes) {
-  (void)rows;
+// blocks working just behind it, even when the vector is larger than L2.  But
+// no more than leaves every resident block an item (launch_slots: the slots of
+// the whole launch): the coarse levels, and whole batches of a few small
+// problems, fitted into 1 to 22 items of 4096 rows, a block each (2 problems of
+// 44^3 with 4 right-hand sides, to 1e-12: 51 -> 9.0 ms; 8 problems of 32^3 to
+// 96^3 with 16: 276 -> 201 ms).
+static int slots_per_item(int64_t launch_slots, int rows_pb, int64_t row_bytes) {
   const int64_t wave = (int64_t)max_grid_blocks();
+  const int64_t fill = std::max<int64_t>(1, launch_slots / wave);
   const int64_t rows_item = std::max<int64_t>(rows_pb, (int64_t(48) << 20) / (wave * std::max<int64_t>(row_bytes, 1)));
-  return (int)std::max<int64_t>(1, std::min<int64_t>(rows_item / rows_pb, 4096 / rows_pb));
+  return (int)std::max<int64_t>(1, std::min<int64_t>({rows_item / rows_pb, 4096 / rows_pb, fill}));
 }
 
 // Resolved tile of one SpMM argument record (as the launcher would pick it).
@@ -175,13 +180,18 @@ static void add_spmm_core(Batch* B, std::vector<BLaunch>& plan, const std::vecto
     std::vector<BItem> items;
     std::vector<BDot> dots;
     size_t smem_d = 0;
+    int64_t launch_slots = 0;
+    for (int i : kv.second) {
+      const int rows_pb = tile_rows_pb(args[i].C / L.cpt, L.kl);
+      launch_slots += ((int64_t)args[i].rows + rows_pb - 1) / rows_pb;
+    }
     for (int i : kv.second) {
       const SpmmArgs& a = args[i];
       const int arg = (int)ga.size();
       ga.push_back(a);
       const int S = (a.C / L.cpt) * L.kl;
       const int rows_pb = tile_rows_pb(a.C / L.cpt, L.kl);
-      const int m = slots_per_item(a.rows, rows_pb, (int64_t)a.C * (xt == VEC_F64 ? 8 : 4));
+      const int m = slots_per_item(launch_slots, rows_pb, (int64_t)a.C * (xt == VEC_F64 ? 8 : 4));
       const int64_t slots = ((int64_t)a.rows + rows_pb - 1) / rows_pb;
       int32_t slot = 0;
       for (int64_t s0 = 0; s0 < slots; s0 += m, ++slot) {
@@ -283,11 +293,16 @@ static void add_vec(Batch* B, std::vector<BLaunch>& plan, int op, VecType vt, co
   std::vector<BItem> items;
   std::vector<BDot> dots;
   size_t smem_d = 0;
+  int64_t launch_slots = 0;
+  for (const UpdArgs& a : args) {
+    const int rows_pb = kBlock / (a.C / cpt);
+    launch_slots += ((int64_t)a.rows + rows_pb - 1) / rows_pb;
+  }
   for (size_t i = 0; i < args.size(); ++i) {
     const UpdArgs& a = args[i];
     const int tpr = a.C / cpt;
     const int rows_pb = kBlock / tpr;
-    const int m = slots_per_item(a.rows, rows_pb, (int64_t)a.C * (vt == VEC_F64 ? 8 : 4));
+    const int m = slots_per_item(launch_slots, rows_pb, (int64_t)a.C * (vt == VEC_F64 ? 8 : 4));
     const int64_t slots = ((int64_t)a.rows + rows_pb - 1) / rows_pb;
     int32_t slot = 0;
     for (int64_t s0 = 0; s0 < slots; s0 += m, ++slot) {
