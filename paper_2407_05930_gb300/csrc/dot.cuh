@@ -95,10 +95,11 @@ __device__ __forceinline__ void dot_finalize_rhs(const DotArgs& d, const double*
 //    columns, not 8 x 5 = 40).
 //  * FP32 partials go to shared memory as they are; kBlock threads sum them as
 //    an unevaluated FP32 pair (error-free additions, the errors summed beside
-//    the sum: 48 bits, the partials themselves carry 24) and convert the pair
-//    once, instead of a conversion and an FP64 add for every partial.
-//  * The block partials: eight loads in flight per thread; from 16 columns on in
-//    two levels, so that the last block does not add nslots x C values alone.
+//    the sum) and convert the pair once, instead of a conversion and an FP64 add
+//    for every partial.  Against exact sums of the 8 to 16 partials of a thread:
+//    off by at most 5e-15 of the sum of magnitudes; a partial itself, by 6e-8.
+//  * The block partials: eight loads in flight per thread; many of them in two
+//    levels, so that the last block does not add nslots x C values alone.
 // Before, from a block's last product to the end of the kernel (456 blocks, FP32):
 // 6.2 us at 8 columns, 12.5 at 24, 10.0 at 32, of which the last block's sum of
 // the block partials 3.0, 6.3 and 7.5; a mixed solve runs three of these an
@@ -302,14 +303,15 @@ __device__ __forceinline__ void block_dot2(const DotArgs& d, DT (&part)[CPT], in
   __syncthreads();  // the block may go on to reuse the shared scratch
 }
 
-// The grid's dot of one problem (slot = block): one level below 16 columns,
-// where the last block's nslots x C adds are shorter than a second arrival.
+// The grid's dot of one problem (slot = block): one level up to 4096 block
+// partials (2 us of FP64 adds in the last block), where a second arrival costs
+// as much as it saves.
 template <int CPT, typename DT>
 __device__ __forceinline__ void block_dot(const DotArgs& d, DT (&part)[CPT], int c0, bool has_cols, int rloc,
                                           int rows_pb, int S, int C, double* sm) {
   const DevScalars& sc = d.sc;
   const int slot = blockIdx.x, nslots = gridDim.x;
-  if (C >= 16 && nslots > 32) {
+  if (nslots * C > 4096 && nslots > 32) {
     BDot bd;
     bd.partials = sc.partials;
     bd.chunk_partials = sc.partials + sc.partial_cap;

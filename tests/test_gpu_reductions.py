@@ -54,3 +54,13 @@ def test_batch_coarsest_solves(nrhs, coarse_max):
     assert all(r.converged for r in res)
     for x, b in zip(xs, bs):
         assert _worst(x, b) <= BOUND
+
+
+@pytest.mark.parametrize("s,nrhs", [(0, 1), (2, 3), (3, 4)])
+def test_pcg_large_magnitudes(s, nrhs):
+    """FP32 partials of 2^90 and more (squares of residuals of 1e15) take the
+    FP64 sums of the fused dots; the same bound holds."""
+    P = amg.Problem.structured(N, 0.0, None, s).setup(coarse_max=40)
+    b = rhs_uniform(P.n, nrhs, config=90 + s) * 1e15
+    x, info = P.solve(torch.from_numpy(b).to("cuda"), tol=1e-12, precision=amg.PREC_MIXED_FP32)
+    assert info.converged and _worst(x, b) <= BOUND
