@@ -25,8 +25,8 @@ constexpr int kJChunk = 8;  // vectors of a set per pass over W
 // of a column combine by the halving exchange of dot.cuh (they swap half of
 // their kJChunk sums), and one barrier per chunk hands the warps' lines to
 // the threads that add them; otherwise every row slot leaves its line.
-__global__ void __launch_bounds__(kBlock) mdot_partial_kernel(const double* __restrict__ V, int64_t vstride,
-                                                              int32_t Cv, int32_t J, const double* __restrict__ W,
+__global__ void __launch_bounds__(kBlock) mdot_partial_kernel(const double* V, int64_t vstride,
+                                                              int32_t Cv, int32_t J, const double* W,
                                                               int64_t rows, int32_t C, double* __restrict__ part) {
   pdl_wait();
   __shared__ double sm[kJChunk * kBlock];  // [line][u][column]
@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(kBlock) mdot_partial_kernel(const double* __re
 // to 608 dependent adds, 110 us a call and two thirds of a GMRES step at 64^3,
 // s = 3; with the exchanges above the solve to 1e-12 went from 22.0 to 12.8 ms.
 constexpr int kFinalCols = 8;
-__global__ void __launch_bounds__(kBlock) mdot_final_kernel(const double* __restrict__ part, int32_t nblk, int32_t n,
+__global__ void __launch_bounds__(kBlock) mdot_final_kernel(const double* part, int32_t nblk, int32_t n,
                                                             double* __restrict__ H) {
   pdl_wait();
   __shared__ double sm[kBlock];
@@ -110,8 +110,8 @@ __global__ void __launch_bounds__(kBlock) mdot_final_kernel(const double* __rest
 }
 
 // W[row][c] += sign * sum_j V_j[row][c % Cv] * H[j * C + c]  (j in order).
-__global__ void __launch_bounds__(kBlock) maxpy_kernel(const double* __restrict__ V, int64_t vstride, int32_t Cv,
-                                                       int32_t J, const double* __restrict__ H, double sign,
+__global__ void __launch_bounds__(kBlock) maxpy_kernel(const double* V, int64_t vstride, int32_t Cv,
+                                                       int32_t J, const double* H, double sign,
                                                        double* __restrict__ W, int64_t rows, int32_t C) {
   pdl_wait();
   const int64_t total = rows * C;
@@ -126,8 +126,8 @@ __global__ void __launch_bounds__(kBlock) maxpy_kernel(const double* __restrict_
 }
 
 // Out[row][c] = W[row][c] * s[c].
-__global__ void __launch_bounds__(kBlock) colscale_kernel(const double* __restrict__ W, const double* __restrict__ s,
-                                                          double* __restrict__ out, int64_t rows, int32_t C) {
+__global__ void __launch_bounds__(kBlock) colscale_kernel(const double* W, const double* s,
+                                                          double* out, int64_t rows, int32_t C) {
   pdl_wait();
   const int64_t total = rows * C;
   for (int64_t e = blockIdx.x * (int64_t)kBlock + threadIdx.x; e < total; e += (int64_t)gridDim.x * kBlock)
@@ -136,8 +136,8 @@ __global__ void __launch_bounds__(kBlock) colscale_kernel(const double* __restri
 
 // out[row][c] = W[row][c] * (1 / sqrt(n2[c])), 0 where n2[c] <= 0: the factors
 // once per block (C <= kBlock).
-__global__ void __launch_bounds__(kBlock) colnormalize_kernel(const double* __restrict__ W,
-                                                              const double* __restrict__ n2, double* __restrict__ out,
+__global__ void __launch_bounds__(kBlock) colnormalize_kernel(const double* W,
+                                                              const double* n2, double* out,
                                                               int64_t rows, int32_t C) {
   pdl_wait();
   __shared__ double s[kBlock];

@@ -124,7 +124,7 @@ __device__ __forceinline__ void butterfly(double (&v)[1 << S]) {
 }
 
 template <int S, int W, typename OT>
-__global__ void __launch_bounds__(kBlock) transform_fwd_kernel(const double* __restrict__ b, int32_t nrhs,
+__global__ void __launch_bounds__(kBlock) transform_fwd_kernel(const double* b, int32_t nrhs,
                                                                int64_t ld, const int32_t* __restrict__ perm,
                                                                int64_t n_b, OT* __restrict__ xhat) {
   pdl_wait();
@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(kBlock) transform_fwd_kernel(const double* __r
 }
 
 template <int S, int W, typename IT>
-__global__ void __launch_bounds__(kBlock) transform_bwd_kernel(const IT* __restrict__ xhat, int32_t nrhs,
+__global__ void __launch_bounds__(kBlock) transform_bwd_kernel(const IT* xhat, int32_t nrhs,
                                                                const int32_t* __restrict__ perm, int64_t n_b,
                                                                double* __restrict__ x, int64_t ld) {
   pdl_wait();
@@ -274,8 +274,8 @@ struct DotAcc<double> {
 
 template <typename T, int CPT, bool HAS_DOT>
 __global__ void __launch_bounds__(kBlock) cg_update1_kernel(int64_t rows, int32_t C, T* __restrict__ x,
-                                                            T* __restrict__ r, const T* __restrict__ p,
-                                                            const T* __restrict__ q, DotArgs dot,
+                                                            T* __restrict__ r, const T* p,
+                                                            const T* q, DotArgs dot,
                                                             const int32_t* skip) {
   pdl_wait();
   using DT = typename DotAcc<T>::type;
@@ -351,7 +351,7 @@ void launch_cg_update1(VecType vt, int64_t rows, int32_t C, void* x, void* r, co
 // p = z + beta p, CPT columns per thread with vector loads.
 template <typename T, int CPT>
 __global__ void __launch_bounds__(kBlock) cg_update2_kernel(int64_t rows, int32_t C, T* __restrict__ p,
-                                                            const T* __restrict__ z, const double* __restrict__ beta,
+                                                            const T* z, const double* beta,
                                                             const int32_t* skip) {
   pdl_wait();
   using V = VecM<T, CPT>;
@@ -407,7 +407,7 @@ void launch_cg_update2(VecType vt, int64_t rows, int32_t C, void* p, const void*
 // One thread per row slice of V columns: z = jd[row] * src (or + z, fused).
 template <typename T, int V>
 __global__ void __launch_bounds__(kBlock) jacobi_kernel(int64_t rows, int32_t C, const T* __restrict__ jd,
-                                                        const T* __restrict__ src, T* z, int accumulate,
+                                                        const T* src, T* z, int accumulate,
                                                         const int32_t* skip) {
   pdl_wait();
   if (skip && *skip == 0) return;
@@ -447,7 +447,7 @@ void launch_jacobi(VecType vt, int64_t rows, int32_t C, const void* jd, const vo
 }
 
 template <typename T>
-__global__ void add_to_f64_kernel(int64_t count, double* __restrict__ y, const T* __restrict__ x) {
+__global__ void add_to_f64_kernel(int64_t count, double* __restrict__ y, const T* x) {
   pdl_wait();
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x)
     y[e] += (double)x[e];
@@ -463,7 +463,7 @@ void launch_add_to_f64(VecType xt, int64_t count, double* y, const void* x, cuda
 }
 
 template <typename T>
-__global__ void copy_kernel(int64_t count, T* __restrict__ d, const T* __restrict__ s) {
+__global__ void copy_kernel(int64_t count, T* __restrict__ d, const T* s) {
   pdl_wait();
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x)
     d[e] = s[e];
@@ -501,8 +501,8 @@ void launch_zero(VecType vt, int64_t count, void* dst, cudaStream_t st) {
 // fraction of its FP32 rate), then the block and grid combine the per-thread
 // partials in FP64 in a fixed order.
 template <typename T, int CPT>
-__global__ void __launch_bounds__(kBlock) dot_kernel(int64_t rows, int32_t C, const T* __restrict__ a,
-                                                     const T* __restrict__ b, DotArgs dot, const int32_t* skip) {
+__global__ void __launch_bounds__(kBlock) dot_kernel(int64_t rows, int32_t C, const T* a,
+                                                     const T* b, DotArgs dot, const int32_t* skip) {
   pdl_wait();
   using DT = typename DotAcc<T>::type;
   using V = VecM<T, CPT>;
@@ -564,13 +564,13 @@ void launch_dot(VecType vt, int64_t rows, int32_t C, const void* a, const void* 
 constexpr int kCoarseBlock = 64;
 template <typename T>
 __global__ void __launch_bounds__(kCoarseBlock) coarse_kernel(int32_t n, int32_t C, const double* __restrict__ Ainv,
-                                                        const T* __restrict__ Y, T* __restrict__ Z,
+                                                        const T* Y, T* __restrict__ Z,
                                                         const int32_t* skip) {
   pdl_wait();
   if (skip && *skip == 0) return;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  coarse_rows_warp<T>(n, C, Ainv, Y, Z, warp, nwarps, [](const auto* p) { return __ldg(p); });
+  coarse_rows_warp<T>(n, C, Ainv, Y, Z, warp, nwarps, [](const auto* p) { return *p; });
 }
 
 void launch_coarse_solve(VecType vt, int32_t n, int32_t C, const double* Ainv, const void* Y, void* Z,
@@ -591,7 +591,7 @@ void launch_coarse_solve(VecType vt, int32_t n, int32_t C, const double* Ainv, c
 // vector is removing the mean of its columns r*nb, r = 0..nrhs-1.
 // Deterministic: per-block partial sums in a fixed tree, one block adds the
 // partials in block order, then the subtraction.
-__global__ void __launch_bounds__(kBlock) block0_partial_kernel(const double* __restrict__ X, int64_t rows,
+__global__ void __launch_bounds__(kBlock) block0_partial_kernel(const double* X, int64_t rows,
                                                                 int32_t C, int32_t nb, int32_t nrhs,
                                                                 double* __restrict__ part) {
   pdl_wait();
@@ -621,7 +621,7 @@ __global__ void block0_mean_kernel(double* part, int32_t nblocks, int32_t nrhs, 
 }
 
 __global__ void __launch_bounds__(kBlock) block0_sub_kernel(double* __restrict__ X, int64_t rows, int32_t C,
-                                                            int32_t nb, int32_t nrhs, const double* __restrict__ mean) {
+                                                            int32_t nb, int32_t nrhs, const double* mean) {
   pdl_wait();
   const int64_t total = rows * nrhs;
   for (int64_t t = blockIdx.x * (int64_t)kBlock + threadIdx.x; t < total; t += (int64_t)gridDim.x * kBlock) {
@@ -653,9 +653,9 @@ void launch_sub_block0_mean(double* X, int64_t rows, int32_t nrhs, int32_t nb, d
 // butterfly) + beta * Z (Z in the output layout; beta = 0 reads no Z),
 // e.g. the residual y - A_c z.
 template <typename T, int NB>
-__global__ void __launch_bounds__(kBlock) coarse_relayout_kernel(const T* __restrict__ in, T* __restrict__ out,
+__global__ void __launch_bounds__(kBlock) coarse_relayout_kernel(const T* in, T* __restrict__ out,
                                                                  int64_t ncb, int32_t nrhs, int dir, double alpha,
-                                                                 double beta, const T* __restrict__ Z) {
+                                                                 double beta, const T* Z) {
   pdl_wait();
   const int64_t total = ncb * nrhs;
   const T scale = dir == 0 ? (T)(alpha / NB) : (T)1;

@@ -10,6 +10,13 @@
 // completion stays transitive along the stream).  Every kernel launched by
 // launch_pdl calls pdl_wait() first, in every thread.
 //
+// The read-only data path (__ldg, or a pointer that is both const and
+// __restrict__) is for data that nothing writes while the kernel lives, and
+// here that life overlaps the predecessor's: it holds for matrices, index lists
+// and the coarsest inverse only.  What another kernel of the solve writes
+// (vectors, dot results, the CG scalars) comes by ordinary loads or through L2,
+// which the wait orders; their pointers carry no __restrict__.
+//
 // Not while a stream is captured: between the kernel nodes of a graph the
 // programmatic edges cost more than they hide (mixed solves 0-2 %, an FP64
 // solve of 87k rows 4 % slower).  Not for a call of a single launch (`pdl` =

@@ -130,7 +130,7 @@ struct ComputeOf<double, double> {
 template <typename MT, typename XT, typename CT, int CPT, bool COH>
 __device__ __forceinline__ void dia_row(const SpmmArgs& a, int row, int c0, CT (&acc)[CPT]) {
   const MT* __restrict__ dv = static_cast<const MT*>(a.dval);
-  const XT* __restrict__ X = static_cast<const XT*>(a.X);
+  const XT* X = static_cast<const XT*>(a.X);
   const int64_t n = a.dstride;
   constexpr int UB = CPT * sizeof(XT) >= 32 ? 4 : kMaxDiag;
 #pragma unroll
@@ -170,7 +170,7 @@ __device__ __forceinline__ void dia_row(const SpmmArgs& a, int row, int c0, CT (
 template <typename MT, typename XT, typename CT, int CPT, int KL, bool COH>
 __device__ __forceinline__ void csr_row(const SpmmArgs& a, int kb, int ke, int e, int c0, CT (&acc)[CPT]) {
   const MT* __restrict__ val = static_cast<const MT*>(a.val);
-  const XT* __restrict__ X = static_cast<const XT*>(a.X);
+  const XT* X = static_cast<const XT*>(a.X);
   const int32_t* __restrict__ idx = a.idx;
   const int C = a.C;
   constexpr int U = CPT >= 8 ? 2 : 4;
@@ -246,7 +246,7 @@ __device__ __forceinline__ void halo_row(const SpmmArgs& a, const XT* xs, int kb
 template <typename XT, typename CT, int CPT, bool COH>
 __device__ __forceinline__ void iface_row(const SpmmArgs& a, int f, int c0, CT (&acc)[CPT]) {
   const CT* __restrict__ iv = static_cast<const CT*>(a.ival);
-  const XT* __restrict__ X = static_cast<const XT*>(a.X);
+  const XT* X = static_cast<const XT*>(a.X);
   for (int ee = __ldg(a.iptr + f); ee < __ldg(a.iptr + f + 1); ++ee) {
     const int j = __ldg(a.icol + ee);
     const Vec<XT, CPT> xv = ldx<XT, CPT, COH>(X + (int64_t)j * a.C + c0);
