@@ -190,7 +190,6 @@ struct SpmmArgs {
   // Early exit: when non-NULL and *skip == 0 (no active RHS) the kernel does
   // nothing (lets the host run one iteration ahead of its convergence check).
   const int32_t* skip = nullptr;
-  bool pdl = true;  // launch_spmm: may start while its predecessor drains (pdl.cuh)
   // Tile: entry lanes per row (1, 2, 4, 8, 16; 0 = 1) and columns per
   // thread (0 = one 16-byte vector; 2x that when C allows); see spmm_kernel.
   int32_t kl = 0;

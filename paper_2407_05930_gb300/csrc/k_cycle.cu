@@ -198,7 +198,9 @@ cudaError_t launch_cycle(ValType mt, VecType vt, int32_t C, int grid, const Cycl
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelExC(&cfg, fn, args);
+  const cudaError_t e = cudaLaunchKernelExC(&cfg, fn, args);
+  pdl_break();
+  return e;
 }
 
 }  // namespace amgsym

@@ -239,6 +239,7 @@ static void launch_h(const SpmmArgs& a, cudaStream_t st) {
   count_launch();
   const int g = std::max(1, std::min(a.htiles, resident_grid((const void*)kern, smem)));
   kern<<<g, kBlock, smem, st>>>(a);
+  pdl_break();
 }
 
 // Blocks that take the flagged (interface) rows while the others run the main
@@ -281,7 +282,7 @@ static void launch_k(const SpmmArgs& a, cudaStream_t st) {
       b.fblocks = iface_blocks(need, nf, &g, res);
     }
     if (dot && (int64_t)g * a.C > a.dot.sc.partial_cap) g = (int)(a.dot.sc.partial_cap / a.C);
-    launch_dep(a.pdl, kern, g, kBlock, smem, st, b);
+    launch_pdl(kern, g, kBlock, smem, st, b);
   };
   if (dot) {
     const size_t smem = sizeof(double) * (size_t)dot_smem_doubles(TPC * KL, rows_pb, a.C);
@@ -314,6 +315,7 @@ static void launch_s(const SpmmArgs& a, cudaStream_t st) {
   const int64_t g = std::max<int64_t>(1, (tasks + kBlock / 32 - 1) / (kBlock / 32));
   if (g > INT32_MAX) fail(AMGSYM_ERR_ARG, "sliced product too large for one launch");
   kern<<<(unsigned)g, kBlock, 0, st>>>(a);
+  pdl_break();
 }
 
 template <typename MT, typename XT, typename OT, int CPT>
@@ -407,6 +409,7 @@ static void launch_zk(const SpmmArgs& a, cudaStream_t st) {
     int g = (int)std::max<int64_t>(1, std::min<int64_t>(resident_grid((const void*)kern, smem), units));
     if (dot && (int64_t)g * a.C > a.dot.sc.partial_cap) g = (int)(a.dot.sc.partial_cap / a.C);
     kern<<<g, kBlock, smem, st>>>(a);
+    pdl_break();
   };
   if constexpr (KM == kKindAll) {
     if (dot && ifc)

@@ -526,6 +526,7 @@ static amgsym_status gmres_impl(amgsym_t h, const double* b_dev, double* x_dev, 
     for (; j < m && total < o.maxit; ++j, ++total) {
       double* vj = V.p + (int64_t)j * len;
       double* zj = Z.p + (int64_t)j * len;
+      PdlScope chain(st);  // the step's launches, up to the copy at its end
       vcycle_apply(c, vj, zj);  // z_j = P v_j (eq. "LRCAMG")
       if (use_lrc) apply_lrc(D, C, zj, part.p, Hd.p, st);
       spmm(c, D->Ainn, VAL_F64, VEC_F64, VEC_F64, zj, w.p, 1.0, 0.0, nullptr, true, nullptr);

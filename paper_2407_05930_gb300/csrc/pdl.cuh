@@ -17,12 +17,21 @@
 // (vectors, dot results, the CG scalars) comes by ordinary loads or through L2,
 // which the wait orders; their pointers carry no __restrict__.
 //
-// Not while a stream is captured: between the kernel nodes of a graph the
+// The attribute goes only to a kernel whose predecessor on the stream is known:
+// a launch_pdl kernel of the same call, with nothing between the two.  A call
+// that is a chain of launches opens a PdlScope on its stream; the first kernel of
+// the scope, and the first after a copy, a memset or a kernel launched otherwise
+// (pdl_break()), starts in the ordinary way, behind whatever the stream holds.  How an early start is ordered
+// behind work that is not a kernel is not documented, so nothing rests on it.
+// Outside a scope every launch is an ordinary one: a setup (its damping decides
+// every later cycle of the handle), a solve (copies between its steps, its
+// iterations in a graph), a batch, and a call of one launch (back-to-back reduced
+// products at 256^3 took 38.6 us with the attribute, 37.0 without).
+//
+// Nor while a stream is captured: between the kernel nodes of a graph the
 // programmatic edges cost more than they hide (mixed solves 0-2 %, an FP64
-// solve of 87k rows 4 % slower).  Not for a call of a single launch (`pdl` =
-// false): back-to-back reduced products at 256^3 took 38.6 us with it, 37.0
-// without.  Eager V-cycles: 57k rows 131 -> 85 us, 256^3 665 -> 612 us; GMRES at
-// 64^3 12.1 -> 11.1 ms.
+// solve of 87k rows 4 % slower).  Eager V-cycles: 57k rows 131 -> 85 us, 256^3
+// 665 -> 612 us; GMRES at 64^3 12.1 -> 11.1 ms.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -36,12 +45,35 @@ __device__ __forceinline__ void pdl_wait() {
   cudaTriggerProgrammaticLaunchCompletion();
 }
 
-template <typename... P, typename... A>
-inline void launch_dep(bool pdl, void (*kern)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, A&&... args) {
-  if (pdl) {
+// The calling thread's open scope.
+struct PdlState {
+  bool on = false;            // an eager stream's scope is open
+  bool after_kernel = false;  // the last operation of the scope was a launch_pdl kernel
+  cudaStream_t st = nullptr;
+};
+extern thread_local PdlState t_pdl;
+
+class PdlScope {
+ public:
+  explicit PdlScope(cudaStream_t st) : outer_(t_pdl) {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    pdl = cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+    const bool eager = cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+    t_pdl = PdlState{eager, false, st};
   }
+  ~PdlScope() { t_pdl = outer_; }
+  PdlScope(const PdlScope&) = delete;
+  PdlScope& operator=(const PdlScope&) = delete;
+
+ private:
+  PdlState outer_;
+};
+
+// After an operation of the scope's stream that is not a launch_pdl kernel.
+inline void pdl_break() { t_pdl.after_kernel = false; }
+
+template <typename... P, typename... A>
+inline void launch_pdl(void (*kern)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, A&&... args) {
+  const bool in_scope = t_pdl.on && t_pdl.st == st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -51,13 +83,9 @@ inline void launch_dep(bool pdl, void (*kern)(P...), dim3 grid, int block, size_
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
+  cfg.numAttrs = in_scope && t_pdl.after_kernel ? 1 : 0;
   (void)cudaLaunchKernelEx(&cfg, kern, P(args)...);  // errors: cudaGetLastError (check_launch)
-}
-
-template <typename... P, typename... A>
-inline void launch_pdl(void (*kern)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, A&&... args) {
-  launch_dep(true, kern, grid, block, smem, st, std::forward<A>(args)...);
+  if (in_scope) t_pdl.after_kernel = true;
 }
 
 }  // namespace amgsym

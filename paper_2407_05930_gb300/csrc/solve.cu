@@ -39,6 +39,7 @@ void check_launch() {
 // Per-launch timing hooks (see Profiler in solver.h).
 
 thread_local Profiler* t_prof = nullptr;
+thread_local PdlState t_pdl;
 
 ProfScope::ProfScope(cudaStream_t st) : st_(st) {
   if (!t_prof) return;
@@ -760,7 +761,6 @@ SpmmArgs make_spmm_args(const Ctx& c, const DevCsr& M, ValType mt, VecType xt, V
   }
   if (dot) a.dot = *dot;
   a.skip = c.skip;
-  a.pdl = c.pdl;
   // the dot-fused variant has its own tile where the tuner timed one
   auto it = c.D->tiles.end();
   if (dot) it = c.D->tiles.find(TileKey{M.idx, c.C, (int)mt, (int)xt, (int)ot, 1});
@@ -1091,6 +1091,7 @@ void prepare_cycle(const Ctx& c) {
   plan.nphases = (int32_t)ph.size();
   plan.phases = dalloc<CyclePhase>(D->work_owned, plan.nphases);
   CK(cudaMemcpy(plan.phases, ph.data(), sizeof(CyclePhase) * ph.size(), cudaMemcpyHostToDevice));
+  pdl_break();
   D->cycle_plans[key] = plan;
 }
 
@@ -1612,7 +1613,6 @@ extern "C" amgsym_status amgsym_apply_reduced(amgsym_t h, const void* X_dev, voi
   const ValType mt = f64 ? VAL_F64 : VAL_F32;
   if (!D->Ainn.vals(mt)) fail(AMGSYM_ERR_STATE, "value precision not built");
   Ctx c{D, nrhs * D->nb, vt, mt, false, (cudaStream_t)stream};
-  c.pdl = false;  // one launch: nothing of this call to overlap
   spmm(c, D->Ainn, mt, vt, vt, X_dev, Y_dev, 1.0, 0.0, nullptr, true, nullptr);
   API_END
 }
@@ -1632,6 +1632,7 @@ extern "C" amgsym_status amgsym_vcycle(amgsym_t h, const void* R_dev, void* Z_de
   Ctx c{D, nrhs * D->nb, vt, mt, finest_hat != 0, (cudaStream_t)stream};
   c.fuse = true;
   prepare_cycle(c);
+  PdlScope chain(c.st);
   vcycle(c, 0, R_dev, Z_dev, nullptr);
   API_END
 }
@@ -1652,6 +1653,7 @@ extern "C" amgsym_status amgsym_amgr_apply(amgsym_t h, const void* R_dev, void* 
   ensure_work(D, nrhs, vt);
   Ctx c{D, nrhs * D->nb, vt, mt, false, (cudaStream_t)stream};
   c.pc = AMGSYM_PC_AMGR;
+  PdlScope chain(c.st);
   amgr_apply(c, R_dev, Z_dev);
   API_END
 }
@@ -1973,6 +1975,7 @@ extern "C" amgsym_status amgsym_vcycle_noalloc(amgsym_t h, const void* R_dev, vo
     }
   }
   Ctx c{D, C, vt, mt, finest_hat != 0, (cudaStream_t)stream};
+  PdlScope chain(c.st);
   vcycle_with(c, lws, 0, R_dev, Z_dev, false);
   API_END
 }

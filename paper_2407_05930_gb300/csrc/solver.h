@@ -182,7 +182,6 @@ struct Ctx {
   const int32_t* skip = nullptr;  // early-exit flag (active RHS count) of the PCG loop
   bool tune = false;              // run the tile autotuner before the first PCG loop
   bool fuse = false;              // coarse levels as one persistent kernel (Device::fuse_level)
-  bool pdl = true;                // programmatic dependent launches (pdl.cuh)
   int pc = AMGSYM_PC_AMG;         // preconditioner of the PCG: the A_inn V-cycle or AMGR
 };
 // The AMGR V-cycle (Alg. "apply"): z = M_AMGR y for every column of c.
