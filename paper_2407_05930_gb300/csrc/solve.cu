@@ -515,8 +515,8 @@ void device_upload(amgsym_problem* p) {
         const uint64_t seed = p->opts.seed + 17 * (uint64_t)l;
         if (V.A.v64 && V.G.v64 && V.Gt.v64)
           L.lambda_max = device_lambda_max(D, V.A, V.G, V.Gt, L.A.rows, seed);
-        else
-          L.lambda_max = lambda_max_GAGt(L.A, L.G, L.Gt, seed);
+        // no eigenvalue of a positive definite matrix: estimated on the host
+        if (!(L.lambda_max > 0.0 && std::isfinite(L.lambda_max))) L.lambda_max = lambda_max_GAGt(L.A, L.G, L.Gt, seed);
         L.omega = (L.lambda_max > 0.0) ? p->opts.omega_scale / L.lambda_max : 1.0;
         V.omega = L.omega;
       }

@@ -68,6 +68,17 @@ def test_new_handles_agree(N, s, nrhs, count):
         P.close()
 
 
+def test_damping_of_a_larger_hierarchy_matches_the_host_estimate():
+    N, s = (128, 112, 96), 3
+    g = gaussian_logk(N, s, seed=35, corr=4.0)
+    P = amg.Problem.structured(N, 1.5, g, s).setup()
+    H = amg.Problem.structured(N, 1.5, g, s).setup(host_only=1)
+    assert P.num_levels() == H.num_levels() >= 4
+    for l in range(P.num_levels() - 1):  # 30 power steps, each to rounding of sums of up to 172k terms
+        w, wh = P.level_info(l)["omega"], H.level_info(l)["omega"]
+        assert abs(w - wh) <= 1e-9 * wh, (l, w, wh)
+
+
 def test_gmres_steps_repeat_bit_for_bit():
     N, s = (32, 32, 32), 3
     P = amg.Problem.structured(N, 1.5, None, s, "neumann").setup(coarse_max=40).lrc_setup(4)
