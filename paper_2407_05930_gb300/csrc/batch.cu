@@ -664,7 +664,7 @@ static amgsym_status batch_solve_impl(Batch* B, const double* const* b_dev, doub
     check_launch();
   }
   int total_it = 0, outer = 0;
-  bool breakdown = false;
+  int broken = -1;  // first problem that broke down
   int64_t relres_off_total = 0;
   for (int p = 0; p < n; ++p) relres_off_total += B->nrhs[p];
   auto read_out = [&](int32_t* any_active) {
@@ -731,10 +731,10 @@ static amgsym_status batch_solve_impl(Batch* B, const double* const* b_dev, doub
       const int32_t* s4 = B->h_status + 4 * n * (1 + (k & 1));
       int32_t act = 0;
       for (int p = 0; p < n; ++p) {
-        if (s4[4 * p + 1]) breakdown = true;
+        if (s4[4 * p + 1] && broken < 0) broken = p;
         act += s4[4 * p];
       }
-      if (breakdown || act == 0) {
+      if (broken >= 0 || act == 0) {
         done_at = k + 1;
         return true;
       }
@@ -760,17 +760,16 @@ static amgsym_status batch_solve_impl(Batch* B, const double* const* b_dev, doub
       launch_add_to_f64(VEC_F32, ctx[p].D->n_b * B->C[p], ctx[p].D->xh, ctx[p].D->w32.x, st);
       check_launch();
     }
-    if (breakdown) break;
+    if (broken >= 0) break;
   }
   for (int p = 0; p < n; ++p) {
     Device* D = ctx[p].D;
     launch_transform_bwd(D->xh, VEC_F64, B->nrhs[p], D->perm, D->n_b, D->s, x_dev[p], B->probs[p]->n, st);
     check_launch();
   }
-  if (breakdown) {
-    BCK(cudaStreamSynchronize(st));
-    fail(AMGSYM_ERR_BREAKDOWN, "PCG breakdown in the batched solve");
-  }
+  if (broken >= 0)
+    fail(AMGSYM_ERR_BREAKDOWN, "PCG breakdown in the batched solve (p^T A p <= 0 or not finite): problem " +
+                                   std::to_string(broken) + ", " + breakdown_text(B->sc_in[broken], st));
   const bool converged = active_out == 0;
   if (infos) {
     BCK(cudaStreamSynchronize(st));

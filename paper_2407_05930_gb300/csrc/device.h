@@ -110,6 +110,7 @@ struct DevScalars {
   double* tol2 = nullptr;    // squared relative-residual target (device scalar)
   int32_t* active = nullptr; // per column: 1 while its RHS has not converged
   int32_t* status = nullptr; // [0] active RHS count, [1] breakdown flag, [2] iterations
+  double* fault = nullptr;   // first breakdown: column, iteration, p^T A p, r^T z (valid with status[1])
   double* partials = nullptr;  // dot-product block partials; chunk sums from partial_cap on
   unsigned* ticket = nullptr;  // last-block counter; the chunks' from 1 on
   int64_t partial_cap = 0;     // doubles available in partials

@@ -26,7 +26,12 @@ __device__ __forceinline__ void dot_finalize_column(const DotArgs& d, int c, dou
       double a = 0.0;
       if (s.active[c] && rz != 0.0) {
         if (sum > 0.0 && isfinite(sum)) a = rz / sum;
-        else s.status[1] = 1;  // breakdown: p^T A p <= 0 or NaN
+        else if (atomicExch(s.status + 1, 1) == 0) {  // breakdown: p^T A p <= 0 or NaN
+          s.fault[0] = c;
+          s.fault[1] = s.status[2];
+          s.fault[2] = sum;
+          s.fault[3] = rz;
+        }
       }
       s.alpha[c] = a;
       break;

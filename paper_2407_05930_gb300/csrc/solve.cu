@@ -10,6 +10,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <cstdio>
 #include <cstring>
 #include <random>
 #include <map>
@@ -599,6 +600,7 @@ void alloc_scalars(Device* D, DevScalars& sc, int32_t C, int32_t nrhs) {
   sc.tol2 = dalloc<double>(D->work_owned, 1);
   sc.active = dalloc<int32_t>(D->work_owned, C);
   sc.status = dalloc<int32_t>(D->work_owned, 4);
+  sc.fault = dalloc<double>(D->work_owned, 4);
   sc.partial_cap = (int64_t)max_grid_blocks() * C;
   // the block partials, then the sums of chunks of 32 blocks; the ticket, then
   // the chunks' (block_dot)
@@ -1392,6 +1394,15 @@ static int pcg_loop(const Ctx& c0, PrecWork& W, const DevScalars& sc, int32_t nr
   return done_at < 0 ? maxit : done_at;
 }
 
+std::string breakdown_text(const DevScalars& sc, cudaStream_t st) {
+  double f[4];
+  CK(cudaMemcpyAsync(f, sc.fault, sizeof(f), cudaMemcpyDeviceToHost, st));
+  CK(cudaStreamSynchronize(st));
+  char t[160];
+  std::snprintf(t, sizeof(t), "column %.0f, iteration %.0f, p^T A p = %.9g, r^T z = %.9g", f[0], f[1], f[2], f[3]);
+  return t;
+}
+
 void check_ptr(const void* p, const char* what) {
   if (!p) fail(AMGSYM_ERR_ARG, std::string(what) + " is NULL");
   if (((uintptr_t)p) % 16) fail(AMGSYM_ERR_ARG, std::string(what) + " must be 16-byte aligned");
@@ -1527,8 +1538,8 @@ static amgsym_status solve_impl(amgsym_t h, const double* b_dev, double* x_dev, 
   launch_transform_bwd(D->xh, VEC_F64, nrhs, D->perm, D->n_b, D->s, x_dev, ld, st);
   check_launch();
   if (breakdown) {
-    CK(cudaStreamSynchronize(st));
-    fail(AMGSYM_ERR_BREAKDOWN, "PCG breakdown (p^T A p <= 0 or not finite)");
+    fail(AMGSYM_ERR_BREAKDOWN, "PCG breakdown (p^T A p <= 0 or not finite): " +
+                                   breakdown_text(mixed ? D->sc_in : D->sc_out, st));
   }
   const bool converged = st4[0] == 0;
   if (!converged) result = AMGSYM_NOT_CONVERGED;

@@ -234,6 +234,8 @@ void spmm(const Ctx& c, const DevCsr& M, ValType mt, VecType xt, VecType ot, con
           double beta, const void* Z, bool iface, const DotArgs* dot);
 DotArgs make_dot(const DevScalars& sc, int mode, int final, const void* W, int32_t nrhs, int32_t nb, double tol,
                  int count_iter);
+// What the kernels saw at the first breakdown of a solve (status[1] set); waits for st.
+std::string breakdown_text(const DevScalars& sc, cudaStream_t st);
 Device* require_dev(amgsym_t h);
 void check_ptr(const void* p, const char* what);
 
