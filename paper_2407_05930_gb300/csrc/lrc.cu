@@ -45,8 +45,8 @@ namespace {
 // Device scratch freed on scope exit.
 struct DevBuf {
   double* p = nullptr;
-  DevBuf() = default;
-  explicit DevBuf(int64_t count) {
+  const int64_t count;
+  explicit DevBuf(int64_t count) : count(count) {
     if (count > 0) CK(cudaMalloc(&p, sizeof(double) * (size_t)count));
   }
   DevBuf(const DevBuf&) = delete;
@@ -110,11 +110,14 @@ void jacobi_eig(std::vector<double>& T, std::vector<double>& Q, int m) {
 }
 
 // z = w + U (Theta V^T w) per column (block c % nb), in place on z.
-void apply_lrc(Device* D, int32_t C, double* z, double* part, double* Hd, cudaStream_t st) {
+void apply_lrc(Device* D, int32_t C, double* z, const DevBuf& part, const DevBuf& Hd, cudaStream_t st) {
   if (D->lrc_k <= 0) return;
+  const int64_t nc = (int64_t)D->lrc_k * C;
+  if (Hd.count < nc || part.count < (int64_t)mdot_blocks(D->n_b, C) * nc)
+    fail(AMGSYM_ERR_STATE, "low-rank correction: the coefficient buffers are too small for its rank");
   const int64_t vs = D->n_b * D->nb;
-  launch_mdot(D->lrc_V, vs, D->nb, D->lrc_k, z, D->n_b, C, part, Hd, st);
-  launch_maxpy(D->lrc_U, vs, D->nb, D->lrc_k, Hd, 1.0, z, D->n_b, C, st);
+  launch_mdot(D->lrc_V, vs, D->nb, D->lrc_k, z, D->n_b, C, part.p, Hd.p, st);
+  launch_maxpy(D->lrc_U, vs, D->nb, D->lrc_k, Hd.p, 1.0, z, D->n_b, C, st);
   check_launch();
 }
 
@@ -474,7 +477,9 @@ static amgsym_status gmres_impl(amgsym_t h, const double* b_dev, double* x_dev, 
   Ctx c{D, C, VEC_F64, VAL_F64, o.finest_hat != 0, st};
   c.fuse = true;
   DevBuf V((int64_t)(m + 1) * len), Z((int64_t)m * len), w(len),
-      part((int64_t)mdot_blocks(n_b, C) * std::max(m + 1, D->lrc_k + 1) * C), Hd((int64_t)(2 * m + 3) * C), sd(C);
+      part((int64_t)mdot_blocks(n_b, C) * std::max(m + 1, D->lrc_k + 1) * C),
+      Hd((int64_t)std::max(2 * m + 3, D->lrc_k) * C),  // a step's two passes and norm; the correction's coefficients
+      sd(C);
   double* bh = D->bh;
   double* xh = D->xh;
   launch_transform_fwd(b_dev, nrhs, ld, D->perm, n_b, D->s, bh, VEC_F64, st);
@@ -528,7 +533,7 @@ static amgsym_status gmres_impl(amgsym_t h, const double* b_dev, double* x_dev, 
       double* zj = Z.p + (int64_t)j * len;
       PdlScope chain(st);  // the step's launches, up to the copy at its end
       vcycle_apply(c, vj, zj);  // z_j = P v_j (eq. "LRCAMG")
-      if (use_lrc) apply_lrc(D, C, zj, part.p, Hd.p, st);
+      if (use_lrc) apply_lrc(D, C, zj, part, Hd, st);
       spmm(c, D->Ainn, VAL_F64, VEC_F64, VEC_F64, zj, w.p, 1.0, 0.0, nullptr, true, nullptr);
       // two Gram-Schmidt passes, the norm and the next basis vector on the
       // device, then one copy of all their coefficients: the host waits once
