@@ -10,6 +10,7 @@
 #pragma once
 
 #include "device.h"
+#include "fp32_sum.h"
 
 namespace amgsym {
 
@@ -98,11 +99,10 @@ __device__ __forceinline__ void dot_finalize_rhs(const DotArgs& d, const double*
 //  * FP64 partials: a warp combines its row slots by halving exchanges (lane
 //    pairs swap half of their columns: 4 + 2 + 1 + 1 + 1 = 9 adds a lane for 8
 //    columns, not 8 x 5 = 40).
-//  * FP32 partials go to shared memory as they are; kBlock threads sum them as
-//    an unevaluated FP32 pair (error-free additions, the errors summed beside
-//    the sum) and convert the pair once, instead of a conversion and an FP64 add
-//    for every partial.  Against exact sums of the 8 to 16 partials of a thread:
-//    off by at most 5e-15 of the sum of magnitudes; a partial itself, by 6e-8.
+//  * FP32 partials go to shared memory as they are; kBlock threads sum up to 16
+//    of them each with error-free FP32 additions (fp32_sum.h: nearer to the exact
+//    sum than additions in FP64) and convert once, instead of a conversion and an
+//    FP64 add for every partial.
 //  * The block partials: eight loads in flight per thread; many of them in two
 //    levels, so that the last block does not add nslots x C values alone.
 // Before, from a block's last product to the end of the kernel (456 blocks, FP32):
@@ -215,9 +215,7 @@ __device__ __forceinline__ void dot_block_sum(double (&part)[CPT], int c0, bool 
   dot_sum_lines<false>(sm, dot_lines(S, rows_pb), C, red, out);
 }
 
-// The same of FP32 partials, as FP32 pairs: hi + x with its exact error (Knuth's
-// two-sum) added to lo.  Partials of 2^90 or more, infinities and NaN are
-// summed in FP64 (the pair could overflow, or turn an infinity into a NaN).
+// The same of FP32 partials (fp32_sum.h).
 template <int CPT>
 __device__ __forceinline__ void dot_block_sum(float (&part)[CPT], int c0, bool has_cols, int rloc, int rows_pb, int S,
                                               int C, double* sm, double* red, double* out) {
@@ -230,25 +228,7 @@ __device__ __forceinline__ void dot_block_sum(float (&part)[CPT], int c0, bool h
   __syncthreads();
   const int nsl = min(kBlock / C, rows_pb);
   const int c = threadIdx.x / nsl, sl = threadIdx.x - c * nsl;
-  if (c < C) {
-    const float* col = f + c * pitch;
-    float hi = 0.f, lo = 0.f;
-    bool big = false;
-    for (int r = sl; r < rows_pb; r += nsl) {
-      const float x = col[r];
-      big |= !(fabsf(x) < 0x1p90f);
-      const float t = __fadd_rn(hi, x);
-      const float xr = __fsub_rn(t, hi);
-      lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, xr)), __fsub_rn(x, xr)));
-      hi = t;
-    }
-    double v = (double)hi + (double)lo;
-    if (big) {
-      v = 0.0;
-      for (int r = sl; r < rows_pb; r += nsl) v += (double)col[r];
-    }
-    red[sl * C + c] = v;
-  }
+  if (c < C) red[sl * C + c] = fp32_sum(f + c * pitch, sl, nsl, rows_pb);
   dot_fold(nsl, C, red, out);
 }
 
