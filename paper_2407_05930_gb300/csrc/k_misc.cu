@@ -410,17 +410,23 @@ __global__ void __launch_bounds__(kBlock) jacobi_kernel(int64_t rows, int32_t C,
                                                         const T* src, T* z, int accumulate,
                                                         const int32_t* skip) {
   pdl_wait();
+  using Vec = VecM<T, V>;
   if (skip && *skip == 0) return;
   const int64_t slices = (int64_t)rows * (C / V);
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < slices; t += (int64_t)gridDim.x * blockDim.x) {
     const int64_t row = t / (C / V);
     const T d = jd[row];
-    const int64_t e = t * V;
+    const Vec s = *reinterpret_cast<const Vec*>(src + t * V);
+    Vec o;
+    if (accumulate) {
+      o = *reinterpret_cast<const Vec*>(z + t * V);
 #pragma unroll
-    for (int q = 0; q < V; ++q) {
-      const T s = src[e + q];
-      z[e + q] = accumulate ? fma(d, s, z[e + q]) : d * s;
+      for (int q = 0; q < V; ++q) o.v[q] = fma(d, s.v[q], o.v[q]);
+    } else {
+#pragma unroll
+      for (int q = 0; q < V; ++q) o.v[q] = d * s.v[q];
     }
+    *reinterpret_cast<Vec*>(z + t * V) = o;
   }
 }
 
