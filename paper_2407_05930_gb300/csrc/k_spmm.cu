@@ -391,11 +391,18 @@ bool spmm_uses_sell(VecType xt, VecType ot, const SpmmArgs& a) {
   return xt == VEC_F64 ? sell_lanes_ok<double>(a.C) : sell_lanes_ok<float>(a.C);
 }
 
+// Two 16-byte vectors of columns a thread move as one 32-byte access, which
+// needs its address aligned to 32 bytes; a caller's vectors are to 16.
+static bool wide_aligned(const SpmmArgs& a) {
+  auto ok = [](const void* p) { return (uintptr_t)p % 32 == 0; };
+  return ok(a.X) && ok(a.Y) && ok(a.Z) && (a.dot.mode != DOT_WY || ok(a.dot.W)) && (a.jmode != 1 || ok(a.Y2));
+}
+
 bool spmm_uses_stencil(ValType mt, VecType xt, VecType ot, const SpmmArgs& a) {
   // FP32 vectors, one thread per row with all 8 columns; the interface only
   // with the full stencil (the reduced operator)
   return a.ndiag > 0 && a.gkm != 0 && xt == VEC_F32 && ot == VEC_F32 && (mt == VAL_F32 || mt == VAL_BF16) &&
-         a.C == 8 && (!a.imask || a.gkm == kKindAll);
+         a.C == 8 && wide_aligned(a) && (!a.imask || a.gkm == kKindAll);
 }
 
 template <typename MT, typename XT, typename OT, int KM>
@@ -443,7 +450,7 @@ static void launch_c(const SpmmArgs& a, cudaStream_t st) {
   }
   // V: elements of the narrower of X / Y in one 16-byte vector
   constexpr int V = 16 / (int)sizeof(XT) < 16 / (int)sizeof(OT) ? 16 / (int)sizeof(XT) : 16 / (int)sizeof(OT);
-  const int want = a.cpt > 0 ? a.cpt : V;
+  const int want = !wide_aligned(a) ? V : a.cpt > 0 ? a.cpt : V;
   if (want >= 2 * V && V == 4 && a.C % 8 == 0 && a.C / 8 <= kBlock)
     launch_t<MT, XT, OT, 8>(a, st);
   else if (want >= 2 * V && V == 2 && a.C % 4 == 0 && a.C / 4 <= kBlock)
@@ -459,7 +466,7 @@ static void launch_c(const SpmmArgs& a, cudaStream_t st) {
 void spmm_resolved_tile(VecType xt, VecType ot, const SpmmArgs& a, int* cpt, int* kl) {
   // the choices of launch_c and launch_t
   const int V = std::min(16 / (xt == VEC_F64 ? 8 : 4), 16 / (ot == VEC_F64 ? 8 : 4));
-  const int want = a.cpt > 0 ? a.cpt : V;
+  const int want = !wide_aligned(a) ? V : a.cpt > 0 ? a.cpt : V;
   int c;
   if (want >= 2 * V && V == 4 && a.C % 8 == 0 && a.C / 8 <= kBlock)
     c = 8;
