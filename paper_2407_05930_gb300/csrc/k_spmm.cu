@@ -90,19 +90,15 @@ __global__ void __launch_bounds__(kBlock, 4) spmm_halo_kernel(SpmmArgs a) {
   extern __shared__ __align__(16) unsigned char halo_smem[];
   XT* xs = reinterpret_cast<XT*>(halo_smem);
   const int C = a.C;
-  const int TPC = C / CPT;
-  const int S = TPC * KL;
-  const int rows_pb = kBlock / S;
-  const int g = threadIdx.x / S;
-  const int w = threadIdx.x - g * S;
-  const int e = KL > 1 ? w / TPC : 0;
-  const int c0 = (w - e * TPC) * CPT;
-  const bool slot_ok = g < rows_pb;
+  constexpr int E = tile_cols<CPT, KL>();
+  const TileLayout lay = tile_layout<CPT, KL>(C);
+  const int rows_pb = lay.rows_pb, g = lay.g, e = lay.e, c0 = lay.c0;
+  const bool slot_ok = lay.slot_ok;
   const int words = C * (int)sizeof(XT) / 4;  // 32-bit words per X row
   const bool vec16 = (words & 3) == 0;
   const int q = vec16 ? words >> 2 : words;   // staged units per X row (16 or 4 bytes)
   const int32_t* __restrict__ ptr = a.ptr;
-  DT dpart[CPT];
+  DT dpart[E];  // (no dot here)
   int t = blockIdx.x;
   int hb_next = 0, he_next = 0;
   if (t < a.htiles) {
@@ -187,16 +183,14 @@ __global__ void __launch_bounds__(kBlock, 4) spmm_halo_kernel(SpmmArgs a) {
         b1 = __ldg(ptr + row + 1);
       }
       if (live) halo_row<MT, XT, CT, CPT, KL>(a, xs, b0, b1, e, c0, acc);
-      if (KL > 1) {
+      combine_lanes<CPT, KL, CT>(lay, acc);
+      if (live && lay.own) {
+        CT out[E];
 #pragma unroll
-        for (int off = KL / 2; off >= 1; off >>= 1) {
-#pragma unroll
-          for (int qq = 0; qq < CPT; ++qq) acc[qq] += __shfl_xor_sync(0xffffffffu, acc[qq], off * TPC);
-        }
+        for (int qq = 0; qq < E; ++qq) out[qq] = acc[qq];
+        row_epilogue<XT, OT, CT, DT, E, false, false>(a, row, lay.ec0, out, Vec<XT, E>{}, false, Vec<XT, E>{}, false,
+                                                      dpart);
       }
-      if (live && e == 0)
-        row_epilogue<XT, OT, CT, DT, CPT, false, false>(a, row, c0, acc, Vec<XT, CPT>{}, false, Vec<XT, CPT>{}, false,
-                                                        dpart);
     }
     __syncthreads();  // the next tile overwrites the halo
   }
@@ -209,12 +203,8 @@ static size_t halo_smem_bytes(VecType xt, const SpmmArgs& a) {
 // The halo form pays off only with tiles enough to fill the GPU: a tile is
 // one block's serial stage-then-compute, so a small level with a few dozen
 // tiles runs faster as the CSR kernel's many short rows.
-// Its row slots are aligned to powers of two within a block.
 bool spmm_uses_halo(VecType xt, const SpmmArgs& a) {
-  int cpt = 0, kl = 0;
-  spmm_resolved_tile(xt, xt, a, &cpt, &kl);
-  const int tpc = a.C / cpt;
-  return (kl == 1 || (tpc & (tpc - 1)) == 0) && a.htiles >= 2 * num_sms() && a.hptr && a.ndiag <= 0 && a.dot.mode == DOT_NONE && !a.imask &&
+  return a.htiles >= 2 * num_sms() && a.hptr && a.ndiag <= 0 && a.dot.mode == DOT_NONE && !a.imask &&
          halo_smem_bytes(xt, a) <= (size_t)kHaloSmemLimit;
 }
 
