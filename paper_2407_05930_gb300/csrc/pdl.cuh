@@ -36,8 +36,6 @@
 
 #include <cuda_runtime.h>
 
-#include <utility>
-
 namespace amgsym {
 
 __device__ __forceinline__ void pdl_wait() {
@@ -71,8 +69,16 @@ class PdlScope {
 // After an operation of the scope's stream that is not a launch_pdl kernel.
 inline void pdl_break() { t_pdl.after_kernel = false; }
 
-template <typename... P, typename... A>
-inline void launch_pdl(void (*kern)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, A&&... args) {
+template <typename T>
+struct Same {
+  using type = T;
+};
+
+// The arguments have the kernel's own parameter types: what is passed converts
+// to them by the language's implicit conversions, checked by the compiler.
+template <typename... P>
+inline void launch_pdl(void (*kern)(P...), dim3 grid, int block, size_t smem, cudaStream_t st,
+                       typename Same<P>::type... args) {
   const bool in_scope = t_pdl.on && t_pdl.st == st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -84,7 +90,7 @@ inline void launch_pdl(void (*kern)(P...), dim3 grid, int block, size_t smem, cu
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = in_scope && t_pdl.after_kernel ? 1 : 0;
-  (void)cudaLaunchKernelEx(&cfg, kern, P(args)...);  // errors: cudaGetLastError (check_launch)
+  (void)cudaLaunchKernelEx(&cfg, kern, args...);  // errors: cudaGetLastError (check_launch)
   if (in_scope) t_pdl.after_kernel = true;
 }
 
