@@ -546,6 +546,7 @@ static amgsym_status gmres_impl(amgsym_t h, const double* b_dev, double* x_dev, 
       }
       double* n2 = Hd.p + 2 * nc;
       launch_mdot(w.p, 0, C, 1, w.p, n_b, C, part.p, n2, st);
+      pdl_break();
       launch_colnormalize(w.p, n2, V.p + (int64_t)(j + 1) * len, n_b, C, st);
       check_launch();
       to_host(hv.data(), Hd.p, 2 * nc + C, st);

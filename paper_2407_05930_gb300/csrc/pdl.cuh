@@ -21,8 +21,11 @@
 // a launch_pdl kernel of the same call, with nothing between the two.  A call
 // that is a chain of launches opens a PdlScope on its stream; the first kernel of
 // the scope, and the first after a copy, a memset or a kernel launched otherwise
-// (pdl_break()), starts in the ordinary way, behind whatever the stream holds.  How an early start is ordered
-// behind work that is not a kernel is not documented, so nothing rests on it.
+// (pdl_break()), starts in the ordinary way, behind whatever the stream holds,
+// and so does the last kernel of a chain, so that what follows the call (a copy, a
+// graph, a caller's kernel) is behind an ordinary launch.  How an early start is
+// ordered before and after work that is not a kernel is not documented; nothing
+// rests on it.
 // Outside a scope every launch is an ordinary one: a setup (its damping decides
 // every later cycle of the handle), a solve (copies between its steps, its
 // iterations in a graph), a batch, and a call of one launch (back-to-back reduced

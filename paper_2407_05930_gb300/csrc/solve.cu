@@ -962,14 +962,16 @@ static void smooth_first(const Ctx& c, const DevLevel& L, LevelWork& lw, const v
 }
 
 static void smooth_sweep(const Ctx& c, const DevLevel& L, LevelWork& lw, const void* y, void* z, bool hat,
-                         const DotArgs* dot) {
+                         const DotArgs* dot, bool ends_cycle = false) {
   level_residual(c, L, z, lw.r, y, hat);
   const void* jd = L.jd(c.vt);
   if (jd && !dot) {
+    if (ends_cycle) pdl_break();
     run_jacobi(c, L, jd, lw.r, z, 1);
     return;
   }
   spmm(c, L.G, c.mt, c.vt, c.vt, lw.r, lw.t, 1.0, 0.0, nullptr, false, nullptr);
+  if (ends_cycle) pdl_break();
   spmm(c, L.Gt, c.mt, c.vt, c.vt, lw.t, z, L.omega, 1.0, z, false, dot);
 }
 
@@ -1180,7 +1182,7 @@ static const void* vcycle_level(const Ctx& c, std::vector<LevelWork>& lws, int l
       run_spmm(c, L.A, mt, vt, vt, a);
       return lw.t;
     }
-    smooth_sweep(c, L, lw, y, z, hat, fin ? last : nullptr);
+    smooth_sweep(c, L, lw, y, z, hat, fin ? last : nullptr, fin && l == 0);
   }
   return z;
 }
@@ -1225,6 +1227,7 @@ void amgr_apply(const Ctx& c, const void* y, void* z) {
   auto smooth = [&](const void* src, double beta) {  // z = beta z + S src
     spmm(c, M.GK, mt, vt, vt, src, W.at, 1.0, 0.0, nullptr, false, nullptr);
     spmm(c, M.GKt, mt, vt, vt, W.at, z, M.omegaK, beta, z, false, nullptr);
+    if (beta != 0.0) pdl_break();  // the last launch
     ProfScope ps(c.st);
     launch_jacobi(vt, D->n_b, c.C, M.jd(vt), src, z, 1, c.st, c.skip);
     check_launch();

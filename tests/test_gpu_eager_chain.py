@@ -52,6 +52,29 @@ def test_chains_equal_captured_ones(N, s, nrhs, prec, form):
     assert all(torch.equal(a, z) for a, z in zip(eager, Z))
 
 
+@pytest.mark.parametrize("prec", [amg.PREC_FP64, amg.PREC_MIXED_FP32])
+@pytest.mark.parametrize("form", ["vcycle", "amgr_apply"])
+def test_a_graph_behind_a_chain_sees_its_result(form, prec):
+    N, s, nrhs = (64, 48, 40), 2, 2
+    g = gaussian_logk(N, s, seed=36, corr=3.0)
+    P = amg.Problem.structured(N, 1.5, g, s).setup(coarse_max=40, amgr=int(form == "amgr_apply"))
+    apply = getattr(P, form)
+    dt = torch.float64 if prec == amg.PREC_FP64 else torch.float32
+    rng = np.random.default_rng(11)
+    R = [torch.from_numpy(rng.uniform(-1.0, 1.0, (P.n_b, nrhs << s))).to(DEV, dt) for _ in range(4)]
+    ref = [apply(r, torch.empty_like(r), nrhs, prec).clone() for r in R]
+    Z, Y = torch.empty_like(R[0]), torch.empty_like(R[0])
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        Y.copy_(Z)
+    for k in range(200):
+        Z.fill_(float("nan"))
+        apply(R[k % 4], Z, nrhs, prec)
+        graph.replay()
+        assert torch.equal(Y, ref[k % 4]), k
+
+
 @pytest.mark.parametrize("N,s,nrhs,count", [((32, 28, 24), 3, 4, 60), ((64, 64, 64), 3, 1, 30)])
 def test_new_handles_agree(N, s, nrhs, count):
     g = gaussian_logk(N, s, seed=34, corr=3.0)
