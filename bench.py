@@ -75,7 +75,9 @@ PROFILED_TRAFFIC = {
 KERNEL_SOURCES = ("paper_2407_05930_gb300/csrc/k_spmm.cu", "paper_2407_05930_gb300/csrc/spmm_common.cuh",
                   "paper_2407_05930_gb300/csrc/k_misc.cu", "paper_2407_05930_gb300/csrc/dot.cuh",
                   "paper_2407_05930_gb300/csrc/stencil.cuh", "paper_2407_05930_gb300/csrc/coarse.cuh",
-                  "paper_2407_05930_gb300/csrc/sell.cuh")
+                  "paper_2407_05930_gb300/csrc/sell.cuh", "paper_2407_05930_gb300/csrc/fp32_sum.h",
+                  "paper_2407_05930_gb300/csrc/pdl.cuh", "paper_2407_05930_gb300/csrc/device.h",
+                  "paper_2407_05930_gb300/csrc/solve.cu")  # the last two choose the tiles
 KERNEL_SOURCES_SHA256 = "c020ba817c60e8ac42ace57ab3db6246cff0b1b6a28686a37ffded62a2d94790"
 
 
