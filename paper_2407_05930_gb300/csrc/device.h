@@ -249,7 +249,7 @@ void spmm_resolved_tile(VecType xt, VecType ot, const SpmmArgs& a, int* cpt, int
 // Whether launch_spmm runs the halo-staged kernel for these arguments.
 bool spmm_uses_halo(VecType xt, const SpmmArgs& a);
 // Whether launch_spmm runs the sliced (SELL) kernel for these arguments.
-bool spmm_uses_sell(VecType xt, VecType ot, const SpmmArgs& a);
+bool spmm_uses_sell(VecType xt, const SpmmArgs& a);
 // Whether launch_spmm runs the z-marching stencil kernel for these arguments.
 bool spmm_uses_stencil(ValType mt, VecType xt, VecType ot, const SpmmArgs& a);
 // The stencil form of a diagonal-offset matrix (offsets off[0..ndiag),

@@ -1,8 +1,9 @@
 // Deterministic per-column dot products fused into kernel epilogues.
 //
-// Every participating kernel uses 256-thread blocks in which thread t owns
-// the CPT consecutive columns c0 = (t % TPR) * CPT of row slot t / TPR.  A
-// block reduces its threads' partials in shared memory in a fixed order,
+// Every participating kernel uses 256-thread blocks in which a thread owns some
+// consecutive columns of a row slot: slot t / TPR for thread t where TPR = C / CPT
+// threads serve a row alone, the place in TileLayout (spmm_common.cuh) in the
+// products.  A block reduces its threads' partials in shared memory in a fixed order,
 // writes one partial per column to global memory, and the last block to
 // finish (integer ticket) sums the block partials in a fixed order and runs
 // the finalisation (CG scalars, convergence test).  No floating-point
@@ -74,7 +75,7 @@ __device__ __forceinline__ void dot_finalize_rhs(const DotArgs& d, const double*
     const double rel2 = bn > 0.0 ? t / bn : 0.0;
     s.relres[r] = sqrt(rel2);
     bool act = s.active[r * nb] != 0;
-    if (act && !(rel2 > *s.tol2)) {  // converged (NaN keeps it active)
+    if (act && !(rel2 > *s.tol2)) {  // converged (or NaN: the breakdown flag was set at p^T A p)
       act = false;
       for (int i = 0; i < nb; ++i) s.active[r * nb + i] = 0;
     }

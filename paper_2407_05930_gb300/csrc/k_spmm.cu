@@ -10,11 +10,11 @@
 //     (Alg. "apply" shape, Sec. 3.2), with epilogues for residuals
 //     (Y = Z - A X) and updates (Y = Z + w G^T X).
 //
-// Layout: X, Y, Z are [rows][C] row-major; thread t of a 256-thread block
-// owns columns c0 = (t % TPR) * CPT .. c0 + CPT - 1 of row slot t / TPR,
-// TPR = C / CPT, so one 16-byte vector load fetches a thread's columns of a
-// neighbour row and the TPR threads of a row read each matrix entry once
-// (broadcast).  Rows are walked grid-stride so a wave of blocks touches a
+// Layout: X, Y, Z are [rows][C] row-major; a row is served by C / CPT column
+// threads (times the entry lanes, see TileLayout), each owning CPT consecutive
+// columns, so one or two 16-byte vectors fetch a thread's columns of a neighbour
+// row and the column threads of a row read each matrix entry once (broadcast).
+// Rows are walked grid-stride so a wave of blocks touches a
 // contiguous window of rows (L2 reuse of the gathered X rows).
 //
 // Matrix storage: CSR, or the diagonal-offset form of a matrix whose
@@ -237,9 +237,10 @@ static void launch_h(const SpmmArgs& a, cudaStream_t st) {
 // column, operand): as a second pass of every block it was a tail of 6 us after
 // the 32 us of the reduced product at 256^3 (FP32), 23 after 99 us in FP64 at
 // 192^3.  One block a slot when everything is resident at once, else their
-// share of the resident blocks, a flagged slot counted as four of the others
-// (counted as two, the flagged rows of the 256^3 product ended last: 39.2 us;
-// now 36.0, 36.9 as a second pass; the FP64 2D 64x64 solve 2.73 -> 2.6 ms).
+// share of the resident blocks, a flagged slot counted as four of the others:
+// measured on the 256^3 product (counted as two, its flagged rows ended last:
+// 39.2 us; now 36.0, 36.9 as a second pass), the same elsewhere (the FP64 2D
+// 64x64 solve 2.73 -> 2.6 ms).
 static int iface_blocks(int64_t slots, int64_t fslots, int* grid, int resident) {
   if (fslots <= 0) return 0;
   if (slots + fslots <= resident) {
@@ -375,9 +376,8 @@ void stencil_geometry(int32_t rows, int32_t ndiag, const int32_t* off, SpmmArgs&
   a.gkm = km;
 }
 
-bool spmm_uses_sell(VecType xt, VecType ot, const SpmmArgs& a) {
+bool spmm_uses_sell(VecType xt, const SpmmArgs& a) {
   if (a.nslices <= 0 || a.ndiag > 0 || a.dot.mode != DOT_NONE || a.imask || spmm_uses_halo(xt, a)) return false;
-  (void)ot;
   return xt == VEC_F64 ? sell_lanes_ok<double>(a.C) : sell_lanes_ok<float>(a.C);
 }
 

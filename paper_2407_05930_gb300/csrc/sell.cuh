@@ -12,17 +12,20 @@
 //
 // Bit-identical to the CSR kernel at the same entry-lane count KL: a row
 // keeps KL partial sums, entry i going to partial i mod KL in ascending
-// order, and combines them in the order of the CSR kernel's xor-shuffle
-// tree ((p0 + p2) + (p1 + p3) for KL = 4), with the same values, gathers,
+// order, and combines them in the order of the CSR kernel's lane exchanges
+// ((p0 + p2) + (p1 + p3) for KL = 4), with the same values, gathers,
 // fma and epilogue.  Padding slots (column -1) are skipped.
 //
-// Selected by opts.sell, off by default: at 256^3 (level 1: 775k rows, 19
-// entries per row) the sliced residual took 100 us against 72 us for the
-// CSR kernel with 4 entry lanes (without the row sorting 115 us; with one
-// row per lane at 8 columns and one wave of blocks 180 us).  ncu of the
-// one-row-per-lane version at 192^3: fewer sectors (8.0M against 10.3M)
-// and instructions (6.5M against 14.8M) than CSR, but long-scoreboard bound
-// at 22 % achieved occupancy.  The FP64 solve gains (254 ms against 282).
+// Selected by opts.sell, off by default.  Against the CSR kernel with the same
+// lanes, 8 columns, residual of level 1 and V-cycle: FP32 at 224^3 (520k rows, 4
+// lanes) 69.5 against 49.7 us and 551 against 413 us, at 96^3 10.1 against 9.7
+// and 153 against 95; FP64 at 224^3 (2 lanes) 198 against 236 us, the V-cycle
+// 1919 against 1860.  With 8 and 16 lanes (short levels) it takes 10 to 39 us
+// where CSR takes 6 to 16.  So only FP64 levels of 100k rows and more gain; the
+// other lanes are there for the option to run, and give the same bits, on every
+// level.  An earlier one-row-per-lane version at 192^3 read fewer sectors (8.0M
+// against 10.3M) and issued fewer instructions (6.5M against 14.8M) than CSR, but
+// was long-scoreboard bound at 22 % achieved occupancy.
 #pragma once
 
 #include "spmm_common.cuh"

@@ -140,7 +140,7 @@ static void run_spmm(const Ctx& c, const DevCsr& M, ValType mt, VecType xt, VecT
   const bool dot = a.dot.mode != DOT_NONE, ifc = a.imask != nullptr, dia = a.ndiag > 0;
   const char* kname = spmm_uses_stencil(mt, xt, ot, a) ? "stencil_kernel<"
                       : spmm_uses_halo(xt, a)                ? "spmm_halo_kernel<"
-                      : spmm_uses_sell(xt, ot, a)            ? "sell_kernel<"
+                      : spmm_uses_sell(xt, a)            ? "sell_kernel<"
                                                              : "spmm_kernel<";
   const std::string kernel = std::string(kname) + tname(mt) + "," + tname(xt) + "," + tname(ot) + "," +
                              std::to_string(cpt) + "," + std::to_string(kl) + "," + (dot ? "1" : "0") + "," +
@@ -672,8 +672,11 @@ void ensure_work(Device* D, int32_t nrhs, VecType vt) {
 // ---------------------------------------------------------------------------
 // Kernel sequencing.
 
-// Fixed tile from the row length and count (the timings of every candidate on
-// hierarchies of 64^3 to 256^3 grids at 8 to 32 columns, GB300).
+// Fixed tile from the row length and count: the timings of every candidate on
+// hierarchies of 64^3 to 256^3 grids at 8 to 32 columns, FP32 and FP64 values, in
+// the single-problem kernels (GB300).  Other column counts, BF16 values and the
+// batched kernels (whose launch bounds differ) take the same rule without
+// timings of their own; opts.tune times them.
 //
 // Columns per thread: two 16-byte vectors in FP32 (a gathered row of 8 columns
 // is one 32-byte sector), and for the diagonal-offset form; one in FP64 CSR

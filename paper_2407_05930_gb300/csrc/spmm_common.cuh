@@ -265,7 +265,7 @@ __device__ __forceinline__ int flag_index(const SpmmArgs& a, int row) {
   return __ldg(a.iprefix + (row >> 5)) + __popc(wd & ((1u << (row & 31)) - 1u));
 }
 
-// Epilogue of one row (entry lane 0): Y = alpha acc + beta Z, the optional dot.
+// Epilogue of CPT columns of one row: Y = alpha acc + beta Z, the optional dot.
 template <typename XT, typename OT, typename CT, typename DT, int CPT, bool HAS_DOT, bool COH>
 __device__ __forceinline__ void row_epilogue(const SpmmArgs& a, int row, int c0, CT (&acc)[CPT],
                                              const Vec<XT, CPT>& zpre, bool use_zpre, const Vec<XT, CPT>& wpre,
@@ -357,7 +357,7 @@ constexpr int spmm_min_blocks() {
 // The KL partial sums of a column combine by halving exchanges: the entry
 // lanes e and e ^ (KL / 2) swap half of their columns and add, then e and
 // e ^ (KL / 4), so a lane ends with E = max(1, CPT / KL) columns from ec0 and
-// runs the epilogue of those (dup: a lower lane holds them).  Against a full
+// runs the epilogue of those (`own`: no lower lane holds them too).  Against a full
 // exchange with the epilogue in lane 0 that is CPT - 1 instead of
 // CPT log2(KL) shuffles and adds, and an epilogue of E instead of CPT columns.
 // Each column's sum is the same tree.  Measured on whole solves to 1e-12 with
