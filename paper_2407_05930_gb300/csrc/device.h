@@ -77,6 +77,7 @@ constexpr int kSellWindow = 256;
 // coupling?) and, per 32-row word, the number of flagged rows before it.
 struct DevIface {
   int32_t n_rows_flagged = 0;
+  int32_t n_runs = 0;          // runs of consecutive flagged rows
   int64_t n_entries = 0;
   uint32_t* mask = nullptr;    // ceil(n_b / 32)
   int32_t* prefix = nullptr;   // ceil(n_b / 32)
@@ -183,7 +184,7 @@ struct SpmmArgs {
   const int32_t* iprefix = nullptr;
   const int32_t* iptr = nullptr;
   const int32_t* irows = nullptr;  // flagged rows, ascending (the second pass)
-  int32_t nflag = 0;
+  int32_t nflag = 0, nruns = 0;
   const int32_t* icol = nullptr;
   const void* ival = nullptr;  // same precision class as the accumulation
   int32_t nb = 1;

@@ -237,17 +237,30 @@ static void launch_h(const SpmmArgs& a, cudaStream_t st) {
 // column, operand): as a second pass of every block it was a tail of 6 us after
 // the 32 us of the reduced product at 256^3 (FP32), 23 after 99 us in FP64 at
 // 192^3.  One block a slot when everything is resident at once, else their
-// share of the resident blocks, a flagged slot counted as four of the others:
-// measured on the 256^3 product (counted as two, its flagged rows ended last:
-// 39.2 us; now 36.0, 36.9 as a second pass), the same elsewhere (the FP64 2D
-// 64x64 solve 2.73 -> 2.6 ms).
-static int iface_blocks(int64_t slots, int64_t fslots, int* grid, int resident) {
+// share of the resident blocks, a flagged slot counted as `weight` of the others.
+//
+// The weight, from timings of 0 (a second pass of every block) and 1 to 12 over
+// grids of 96^3 to 256^3 and 2D ones with 1 to 3 mirror planes and 2 to 256
+// columns.  FP64 products are bound by FP64 issue, so a flagged row costs its
+// couplings more, 5/4: at 256^3 290 us for 8 columns (290 as a second pass, 308
+// with a weight of 4), at 96^3 581 -> 499 us for 256 columns.  FP32 products are
+// bound by sectors.  Flagged rows that follow one another share theirs; an
+// isolated one (a plane normal to the fastest axis) fetches its values, operands
+// and neighbours alone.  3/2 with a run's start counting 9/2 more: 3 for the three
+// planes of a cube (256^3: 35.5 us, 37.1 as a second pass, 36.8 with 4), 6 for the
+// one strided plane of s = 1 (192^3, 8 columns: 59.3 us, 59.7 as a second pass,
+// 61.2 with 4).
+static double iface_weight(bool f64, int32_t nflag, int32_t nruns) {
+  return f64 ? 1.25 : 1.5 + 4.5 * (double)nruns / (double)nflag;
+}
+
+static int iface_blocks(int64_t slots, int64_t fslots, double weight, int* grid, int resident) {
   if (fslots <= 0) return 0;
   if (slots + fslots <= resident) {
     *grid = (int)(slots + fslots);
     return (int)fslots;
   }
-  const int64_t share = (int64_t)*grid * 4 * fslots / (slots + 4 * fslots);
+  const int64_t share = (int64_t)((double)*grid * weight * (double)fslots / ((double)slots + weight * (double)fslots) + 0.5);
   return (int)std::max<int64_t>(1, std::min<int64_t>(share, *grid / 2));
 }
 
@@ -270,7 +283,7 @@ static void launch_k(const SpmmArgs& a, cudaStream_t st) {
       const int64_t nf = ((int64_t)a.nflag + rows_pb - 1) / rows_pb;
       if (need + nf > res) g = std::max(2, res);
       if (dot && (int64_t)g * a.C > a.dot.sc.partial_cap) g = (int)(a.dot.sc.partial_cap / a.C);
-      b.fblocks = iface_blocks(need, nf, &g, res);
+      b.fblocks = iface_blocks(need, nf, iface_weight(sizeof(XT) == 8, a.nflag, a.nruns), &g, res);
     }
     if (dot && (int64_t)g * a.C > a.dot.sc.partial_cap) g = (int)(a.dot.sc.partial_cap / a.C);
     launch_pdl(kern, g, kBlock, smem, st, b);

@@ -257,6 +257,7 @@ static DevIface upload_iface(std::vector<void*>& owner, int64_t rows, const std:
     run += __builtin_popcount(mask[w]);
   }
   F.n_rows_flagged = run;
+  for (size_t f = 0; f < irows.size(); ++f) F.n_runs += f == 0 || irows[f] != irows[f - 1] + 1;
   F.n_entries = ne;
   F.mask = upload(owner, mask.data(), words);
   F.prefix = upload(owner, prefix.data(), words);
@@ -733,6 +734,7 @@ SpmmArgs make_spmm_args(const Ctx& c, const DevCsr& M, ValType mt, VecType xt, V
     a.iptr = c.D->iface.iptr;
     a.irows = c.D->iface.irows;
     a.nflag = c.D->iface.n_rows_flagged;
+    a.nruns = c.D->iface.n_runs;
     a.icol = c.D->iface.icol;
     const bool f64 = (mt == VAL_F64) || (xt == VEC_F64);
     a.ival = f64 ? (const void*)c.D->iface.ival64 : (const void*)c.D->iface.ival32;
@@ -937,6 +939,7 @@ static void level_residual(const Ctx& c, const DevLevel& L, const void* z, void*
       a.iptr = S.iface.iptr;
       a.irows = S.iface.irows;
       a.nflag = S.iface.n_rows_flagged;
+      a.nruns = S.iface.n_runs;
       a.icol = S.iface.icol;
       a.ival = (c.mt == VAL_F64 || c.vt == VEC_F64) ? (const void*)S.iface.ival64 : (const void*)S.iface.ival32;
       a.nb = S.nb;
