@@ -103,6 +103,7 @@ __device__ __forceinline__ TrVec<T, W> tr_load(const T* p) {
 static __device__ __noinline__ double scale_product(double v, double f) { return v * f; }
 template <int S>
 __device__ __forceinline__ double scale_down(double v) {
+  if constexpr (S == 0) return v;
   const int hi = __double2hiint(v);
   const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;
   if (e - (S + 1u) < 0x7ffu - (S + 1u)) return __hiloint2double(hi - (S << 20), __double2loint(v));
@@ -123,6 +124,26 @@ __device__ __forceinline__ void butterfly(double (&v)[1 << S]) {
   }
 }
 
+// body(r, l) for every right-hand side and base cell.  Each right-hand side has
+// blocks of its own: 2^s gathers a thread are work enough, and a grid cut to about
+// one wave left its last blocks to a second one (96^3, s = 3, 32 right-hand sides
+// 183 -> 168 us).  Without symmetries a thread's share is one value, and one wave
+// of blocks walks all of them (40^3, 32 right-hand sides: 15.6 us, 17.3 with blocks
+// for each right-hand side).
+template <int S, typename F>
+__device__ __forceinline__ void transform_each(int64_t n_b, int32_t nrhs, F&& body) {
+  const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+  if constexpr (S == 0) {
+    for (int64_t t = t0; t < n_b * nrhs; t += step) {
+      const int64_t r = t / n_b;
+      body((int)r, t - r * n_b);
+    }
+  } else {
+    for (int r = blockIdx.y; r < nrhs; r += gridDim.y)
+      for (int64_t l = t0; l < n_b; l += step) body(r, l);
+  }
+}
+
 template <int S, int W, typename OT>
 __global__ void __launch_bounds__(kBlock) transform_fwd_kernel(const double* b, int32_t nrhs,
                                                                int64_t ld, const int32_t* __restrict__ perm,
@@ -130,22 +151,20 @@ __global__ void __launch_bounds__(kBlock) transform_fwd_kernel(const double* b, 
   pdl_wait();
   constexpr int NB = 1 << S;
   const int64_t C = (int64_t)nrhs * NB;
-  for (int r = blockIdx.y; r < nrhs; r += gridDim.y) {
-    for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < n_b; l += (int64_t)gridDim.x * blockDim.x) {
-      double v[NB];
+  transform_each<S>(n_b, nrhs, [&](int r, int64_t l) {
+    double v[NB];
 #pragma unroll
-      for (int j = 0; j < NB; ++j) v[j] = __ldcs(b + r * ld + __ldcs(perm + j * n_b + l));
-      butterfly<S>(v);
-      OT* o = xhat + l * C + r * NB;
+    for (int j = 0; j < NB; ++j) v[j] = __ldcs(b + r * ld + __ldcs(perm + j * n_b + l));
+    butterfly<S>(v);
+    OT* o = xhat + l * C + r * NB;
 #pragma unroll
-      for (int i = 0; i < NB; i += W) {
-        TrVec<OT, W> t;
+    for (int i = 0; i < NB; i += W) {
+      TrVec<OT, W> t;
 #pragma unroll
-        for (int q = 0; q < W; ++q) t.v[q] = (OT)v[i + q];
-        tr_store<OT, W>(o + i, t);
-      }
+      for (int q = 0; q < W; ++q) t.v[q] = (OT)v[i + q];
+      tr_store<OT, W>(o + i, t);
     }
-  }
+  });
 }
 
 template <int S, int W, typename IT>
@@ -155,24 +174,22 @@ __global__ void __launch_bounds__(kBlock) transform_bwd_kernel(const IT* xhat, i
   pdl_wait();
   constexpr int NB = 1 << S;
   const int64_t C = (int64_t)nrhs * NB;
-  for (int r = blockIdx.y; r < nrhs; r += gridDim.y) {
-    for (int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; l < n_b; l += (int64_t)gridDim.x * blockDim.x) {
-      double v[NB];
-      int32_t to[NB];
-      const IT* in = xhat + l * C + r * NB;
+  transform_each<S>(n_b, nrhs, [&](int r, int64_t l) {
+    double v[NB];
+    int32_t to[NB];
+    const IT* in = xhat + l * C + r * NB;
 #pragma unroll
-      for (int i = 0; i < NB; i += W) {
-        const TrVec<IT, W> t = tr_load<IT, W>(in + i);
+    for (int i = 0; i < NB; i += W) {
+      const TrVec<IT, W> t = tr_load<IT, W>(in + i);
 #pragma unroll
-        for (int q = 0; q < W; ++q) v[i + q] = (double)t.v[q];
-      }
-#pragma unroll
-      for (int j = 0; j < NB; ++j) to[j] = __ldcs(perm + j * n_b + l);
-      butterfly<S>(v);
-#pragma unroll
-      for (int j = 0; j < NB; ++j) __stcs(x + r * ld + to[j], scale_down<S>(v[j]));
+      for (int q = 0; q < W; ++q) v[i + q] = (double)t.v[q];
     }
-  }
+#pragma unroll
+    for (int j = 0; j < NB; ++j) to[j] = __ldcs(perm + j * n_b + l);
+    butterfly<S>(v);
+#pragma unroll
+    for (int j = 0; j < NB; ++j) __stcs(x + r * ld + to[j], scale_down<S>(v[j]));
+  });
 }
 
 // Values per vector: the widest of 32 bytes or less that a thread's 2^S values
@@ -190,15 +207,15 @@ static void transform_width(const void* xhat, F&& run) {
     run(std::integral_constant<int, 1>{});
 }
 
-static dim3 transform_grid(int64_t n_b, int32_t nrhs) {
-  const int64_t gx = std::max<int64_t>(1, std::min<int64_t>((n_b + kBlock - 1) / kBlock, max_grid_blocks()));
-  return dim3((unsigned)gx, (unsigned)std::max<int64_t>(1, std::min<int64_t>(nrhs, (max_grid_blocks() + gx - 1) / gx)));
+static dim3 transform_grid(int s, int64_t n_b, int32_t nrhs) {
+  if (s == 0) return dim3((unsigned)grid_for(n_b * nrhs, kBlock));
+  return dim3((unsigned)grid_for(n_b, kBlock), (unsigned)std::min<int32_t>(nrhs, 65535));
 }
 
 template <typename OT>
 static void fwd_dispatch(const double* b, int32_t nrhs, int64_t ld, const int32_t* perm, int64_t n_b, int32_t s,
                          OT* xhat, cudaStream_t st) {
-  const dim3 g = transform_grid(n_b, nrhs);
+  const dim3 g = transform_grid(s, n_b, nrhs);
   auto go = [&](auto sc) {
     constexpr int S = decltype(sc)::value;
     transform_width<S, OT>(xhat, [&](auto w) {
@@ -227,7 +244,7 @@ void launch_transform_fwd(const double* b, int32_t nrhs, int64_t ld, const int32
 template <typename IT>
 static void bwd_dispatch(const IT* xhat, int32_t nrhs, const int32_t* perm, int64_t n_b, int32_t s, double* x,
                          int64_t ld, cudaStream_t st) {
-  const dim3 g = transform_grid(n_b, nrhs);
+  const dim3 g = transform_grid(s, n_b, nrhs);
   auto go = [&](auto sc) {
     constexpr int S = decltype(sc)::value;
     transform_width<S, IT>(xhat, [&](auto w) {
