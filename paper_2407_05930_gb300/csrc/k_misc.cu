@@ -488,8 +488,18 @@ void launch_add_to_f64(VecType xt, int64_t count, double* y, const void* x, cuda
 template <typename T>
 __global__ void copy_kernel(int64_t count, T* __restrict__ d, const T* s) {
   pdl_wait();
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x)
-    d[e] = s[e];
+  // four loads in flight before the stores: 21 us for 2 x 67 MB, 33 with one
+  constexpr int U = 4;
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < count; e += U * step) {
+    T v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (e + u * step < count) v[u] = s[e + u * step];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (e + u * step < count) d[e + u * step] = v[u];
+  }
 }
 
 void launch_copy(VecType vt, int64_t count, void* dst, const void* src, cudaStream_t st) {
